@@ -37,11 +37,6 @@ int limb_max_m(int delta, int n);                                         // sk_
 int finalize_count(int variant, int n, int convention, int nprimes, const uint64_t* primes,
                    const uint64_t* H, sk_u128* out);                      // sk_host_exact.cu
 
-struct BatchScratch {
-  unsigned long long counter;   // next chunk
-  unsigned int err;
-  unsigned int pad;
-};
 
 __device__ __forceinline__ Res4 batch_dispatch(int code, const BatchJobDev* j, const Primes* P,
                                                int np, unsigned long long it, signed char* ws) {
@@ -63,7 +58,7 @@ __device__ __forceinline__ Res4 batch_dispatch(int code, const BatchJobDev* j, c
 
 __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
     batch_kernel(const BatchJobDev* __restrict__ jobs, int njobs, unsigned long long total_chunks,
-                 const Primes* P, int nprimes, BatchScratch* scr, unsigned long long* res) {
+                 const Primes* P, int nprimes, unsigned long long* counter, ExactScratch* sums) {
   extern __shared__ signed char sk_ws[];
   const int lane = threadIdx.x & 31;
   signed char* ws_col = sk_ws + threadIdx.x;
@@ -71,7 +66,7 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
   int cur = -1;
   for (;;) {
     unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(&scr->counter, 1ULL);
+    if (lane == 0) c = atomicAdd(counter, 1ULL);
     c = __shfl_sync(0xffffffffu, c, 0);
     if (c >= total_chunks) break;
     int lo = 0, hi = njobs - 1;                  // last job with chunk_lo <= c
@@ -81,7 +76,7 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
       else hi = mid - 1;
     }
     if (lo != cur) {
-      if (cur >= 0) warp_flush(tot, nprimes, *P, res + (size_t)cur * kMaxPrimes, &scr->err);
+      if (cur >= 0) warp_flush(tot, nprimes, *P, sums + cur);
       cur = lo;
     }
     const BatchJobDev* j = &jobs[lo];
@@ -91,7 +86,7 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
     for (int i = 0; i < kMaxPrimes; ++i)
       if (i < nprimes) tot[i] = addmod(tot[i], r.r[i], (unsigned long long)P->pr[i].p);
   }
-  if (cur >= 0) warp_flush(tot, nprimes, *P, res + (size_t)cur * kMaxPrimes, &scr->err);
+  if (cur >= 0) warp_flush(tot, nprimes, *P, sums + cur);
 }
 
 }  // namespace sk
@@ -312,11 +307,10 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
     if (w > max_ws) max_ws = w;
   }
   const unsigned long long total_chunks = chunk;
-  // device layout: jobs | primes | batch scratch | residues | per-job scratch
+  // device layout: jobs | primes | chunk counter | per-job sums
   const size_t off_p = (sizeof(BatchJobDev) * njobs + 255) / 256 * 256;
   const size_t off_s = off_p + (sizeof(Primes) + 255) / 256 * 256;
-  const size_t off_r = off_s + 256;
-  const size_t off_j = off_r + ((size_t)njobs * kMaxPrimes * 8 + 255) / 256 * 256;
+  const size_t off_j = off_s + 256;
   const size_t bytes = off_j + sizeof(ExactScratch) * (size_t)njobs;
   const size_t out_bytes = bytes - off_s;           // what comes back to the host
   cudaStream_t s = (o && o->stream) ? (cudaStream_t)o->stream : nullptr;
@@ -355,8 +349,8 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
     if (mode == SK_BATCH_PERSISTENT) {
       batch_kernel<<<grid, bt, smem, s>>>((const BatchJobDev*)dbuf, njobs, total_chunks,
                                           (const Primes*)(dbuf + off_p), k,
-                                          (BatchScratch*)(dbuf + off_s),
-                                          (unsigned long long*)(dbuf + off_r));
+                                          (unsigned long long*)(dbuf + off_s),
+                                          (ExactScratch*)(dbuf + off_j));
       r = cudaGetLastError();
     } else {
       launches = 0;
@@ -403,18 +397,12 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
     if (ms < kms_min) kms_min = ms;
   }
   if (e == cudaSuccess) {
-    const BatchScratch* hs = (const BatchScratch*)hbuf;
-    const unsigned long long* hr = (const unsigned long long*)(hbuf + (off_r - off_s));
     const ExactScratch* hjs = (const ExactScratch*)(hbuf + (off_j - off_s));
-    bool err = mode == SK_BATCH_PERSISTENT ? hs->err != 0 : false;
-    for (int q = 0; q < njobs; ++q)
-      if (mode == SK_BATCH_PER_JOB && hjs[q].err) err = true;
-    if (err) st = SK_ETIMEOUT;
     for (int q = 0; q < njobs && !st; ++q) {
       const int j = order[q];
       uint64_t H[kMaxPrimes] = {0, 0, 0, 0};
       for (int i = 0; i < k; ++i)
-        H[i] = mode == SK_BATCH_PERSISTENT ? hr[(size_t)q * kMaxPrimes + i] : hjs[q].res[i];
+        H[i] = scratch_residue(hjs[q], i, pv[i]);
       const int sj = finalize_count(plan[j].variant, plan[j].n, conv, k, pv, H, &outs[j]);
       if (status) status[j] = sj;
       if (sj) st = SK_EMISMATCH;

@@ -50,10 +50,14 @@ inline int device_sm_count(int dev) {
 // Scratch words of one launch (device memory, zeroed before the launch).
 struct ExactScratch {
   unsigned long long counter;            // next chunk of items
-  unsigned long long res[kMaxPrimes];    // residues of the sum, raw
-  unsigned int err;                      // nonzero: a bounded loop gave up
-  unsigned int pad;
+  unsigned long long lo[kMaxPrimes];     // sums of the residues' low 32 bits,
+  unsigned long long hi[kMaxPrimes];     // and of the bits above
 };
+
+// Residue i of a launch, on the host.
+inline unsigned long long scratch_residue(const ExactScratch& h, int i, unsigned long long p) {
+  return (unsigned long long)((((unsigned __int128)h.hi[i] << 32) + h.lo[i]) % p);
+}
 
 struct ExactLaunch {
   ExactJob job;
@@ -68,8 +72,6 @@ struct ExactLaunch {
   cudaStream_t stream;
 };
 
-constexpr int kCasLimit = 1 << 22;
-
 // Two resident 256-thread CTAs per SM: 128 registers per thread, which holds
 // the n correlations, the window of outer values and the accumulators
 // without spills.
@@ -77,22 +79,12 @@ constexpr int kCasLimit = 1 << 22;
 #define SK_EXACT_MIN_BLOCKS 2
 #endif
 
-__device__ __forceinline__ void atomic_addmod(unsigned long long* addr, unsigned long long v,
-                                              unsigned long long p, unsigned int* err) {
-  if (v == 0) return;
-  unsigned long long old = *((volatile unsigned long long*)addr);
-  for (int it = 0; it < kCasLimit; ++it) {
-    unsigned long long nv = addmod(old, v, p);
-    unsigned long long seen = atomicCAS(addr, old, nv);
-    if (seen == old) return;
-    old = seen;
-  }
-  atomicOr(err, 1u);
-}
-
+// Adds the warp's residues to the sums of a launch (or of one job of a
+// batch) and clears them.  Two plain additions a modulus: a compare-and-swap
+// modular add costs a try per competing warp, 1.4 ms when the 2400 warps of a
+// full grid finish together.
 __device__ __forceinline__ void warp_flush(unsigned long long (&tot)[kMaxPrimes], int nprimes,
-                                           const Primes& P, unsigned long long* slots,
-                                           unsigned int* err) {
+                                           const Primes& P, ExactScratch* scr) {
 #pragma unroll
   for (int i = 0; i < kMaxPrimes; ++i) {
     if (i >= nprimes) break;
@@ -100,7 +92,10 @@ __device__ __forceinline__ void warp_flush(unsigned long long (&tot)[kMaxPrimes]
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
       v = addmod(v, __shfl_xor_sync(0xffffffffu, v, o), (unsigned long long)P.pr[i].p);
-    if ((threadIdx.x & 31) == 0) atomic_addmod(&slots[i], v, (unsigned long long)P.pr[i].p, err);
+    if ((threadIdx.x & 31) == 0 && v) {
+      atomicAdd(&scr->lo[i], v & 0xffffffffULL);
+      atomicAdd(&scr->hi[i], v >> 32);
+    }
     tot[i] = 0;
   }
 }
@@ -169,7 +164,7 @@ __device__ __forceinline__ void work_loop(const ExactJob& job, const Primes& P, 
       }
     }
   }
-  warp_flush(tot, nprimes, P, scr->res, &scr->err);
+  warp_flush(tot, nprimes, P, scr);
 }
 
 template <int DELTA, int N>

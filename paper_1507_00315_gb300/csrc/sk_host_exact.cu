@@ -364,8 +364,7 @@ static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long h
   float ms = 0.f;
   cudaEventElapsedTime(&ms, e0, e1);
   *kernel_ms += ms;
-  if (h.err) return SK_ETIMEOUT;
-  for (int i = 0; i < pl.nprimes; ++i) res[i] = h.res[i];
+  for (int i = 0; i < pl.nprimes; ++i) res[i] = scratch_residue(h, i, pl.primes[i]);
   if (grid_used) *grid_used = pl.grid;
   return SK_OK;
 }
