@@ -22,6 +22,7 @@ LIB = os.path.join(PKG, "libskolem.so")
 MAX_N = 31
 MAX_IE_N = 24          # kMaxIeN of csrc/sk_ie.cuh: orders with an inclusion-exclusion kernel
 MIN_MIRROR_N = 6       # kMirrorMinN of csrc/sk_mirror.cuh: orders with a mirrored (Lemma 2.3) kernel
+MIN_SPARSE_N = 13      # kSparseMinN of csrc/sk_sparse.cuh: orders of the zero-skipping walk (mirrored too)
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # Relocatable device code: the batch kernel calls the per-n walk functions
@@ -59,7 +60,9 @@ def _sources():
                 f'SK_INSTANTIATE_EXACT({n})\nSK_DEFINE_BATCH({n})\n')
         if n <= MAX_IE_N:
             text += f'#include "sk_ie.cuh"\nSK_INSTANTIATE_IE({n})\n'
-        if n >= MIN_MIRROR_N:
+        if n >= MIN_SPARSE_N:
+            text += f'#include "sk_sparse.cuh"\nSK_INSTANTIATE_SPARSE({n})\n'
+        elif n >= MIN_MIRROR_N:
             text += f'#include "sk_mirror.cuh"\nSK_INSTANTIATE_MIRROR({n})\n'
         if not os.path.exists(p) or open(p).read() != text:
             with open(p, "w") as f:

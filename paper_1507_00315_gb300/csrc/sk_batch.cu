@@ -39,10 +39,10 @@ int finalize_count(int variant, int n, int convention, int nprimes, const uint64
 
 
 __device__ __forceinline__ Res4 batch_dispatch(int code, const BatchJobDev* j, const Primes* P,
-                                               int np, unsigned long long it, signed char* ws) {
+                                               int np, unsigned long long c, const BatchSmem& sm) {
 #define SK_BCASE(N)                                     \
-  case N: return SK_BATCH_FN(0, N)(j, P, np, it, ws);   \
-  case 32 + N: return SK_BATCH_FN(1, N)(j, P, np, it, ws);
+  case N: return SK_BATCH_FN(0, N)(j, P, np, c, sm);    \
+  case 32 + N: return SK_BATCH_FN(1, N)(j, P, np, c, sm);
   switch (code) {
     SK_BCASE(1) SK_BCASE(2) SK_BCASE(3) SK_BCASE(4) SK_BCASE(5) SK_BCASE(6) SK_BCASE(7)
     SK_BCASE(8) SK_BCASE(9) SK_BCASE(10) SK_BCASE(11) SK_BCASE(12) SK_BCASE(13) SK_BCASE(14)
@@ -58,10 +58,20 @@ __device__ __forceinline__ Res4 batch_dispatch(int code, const BatchJobDev* j, c
 
 __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
     batch_kernel(const BatchJobDev* __restrict__ jobs, int njobs, unsigned long long total_chunks,
-                 const Primes* P, int nprimes, unsigned long long* counter, ExactScratch* sums) {
-  extern __shared__ signed char sk_ws[];
+                 const Primes* P, int nprimes, unsigned long long* counter, ExactScratch* sums,
+                 int sparse) {
+  // the zero-skipping walk's tables and per-warp areas (sparse: some job
+  // uses them), then the dense walk's columns
+  extern __shared__ __align__(16) unsigned char sk_batch_smem[];
   const int lane = threadIdx.x & 31;
-  signed char* ws_col = sk_ws + threadIdx.x;
+  BatchSmem sm;
+  const int warps = blockDim.x >> 5;
+  const int dense = sparse ? sp_table_bytes(0) + warps * kSpWarp : 0;
+  sm.tab = (unsigned)__cvta_generic_to_shared(sk_batch_smem);
+  sm.wsm = sm.tab + sp_table_bytes(0) + (threadIdx.x >> 5) * kSpWarp;
+  sm.ws_col = (signed char*)sk_batch_smem + dense + threadIdx.x;
+  if (sparse) sp_build_tables<0>(sk_batch_smem);
+  __syncthreads();
   unsigned long long tot[kMaxPrimes] = {0, 0, 0, 0};
   int cur = -1;
   for (;;) {
@@ -80,8 +90,7 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
       cur = lo;
     }
     const BatchJobDev* j = &jobs[lo];
-    const unsigned long long item = (c - j->chunk_lo) * 32ULL + (unsigned long long)lane;
-    const Res4 r = batch_dispatch(j->code, j, P, nprimes, item, ws_col);
+    const Res4 r = batch_dispatch(j->code, j, P, nprimes, c - j->chunk_lo, sm);
 #pragma unroll
     for (int i = 0; i < kMaxPrimes; ++i)
       if (i < nprimes) tot[i] = addmod(tot[i], r.r[i], (unsigned long long)P->pr[i].p);
@@ -289,22 +298,54 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   std::stable_sort(order.begin(), order.end(),
                    [&](int a, int b) { return plan[a].terms > plan[b].terms; });
   std::vector<BatchJobDev> hj(njobs);
-  unsigned long long chunk = 0, terms = 0;
-  int max_ws = 0;
+  unsigned long long terms = 0, item_chunks = 0, tiles = 0;
+  int max_ws = 0, sparse = 0;
   for (int r = 0; r < njobs; ++r) {
     const JobPlan& J = plan[order[r]];
     BatchJobDev& d = hj[r];
     std::memset(&d, 0, sizeof(d));
     d.pres = position_mask(J.variant, J.n);
     d.items = J.items;
-    d.chunk_lo = chunk;
-    d.chunks = (J.items + 31) / 32;
     d.m = J.m;
     d.code = J.delta * 32 + J.n;
-    chunk += d.chunks;
     terms += J.terms;
-    const int w = ws_len(J.delta, J.n);
-    if (w > max_ws) max_ws = w;
+    item_chunks += (J.items + 31) / 32;
+    if (J.n >= kSparseMinN) {
+      if (!sp_plain_job(d.pres, J.delta, J.n, J.m, 0, 0, J.items, &d.sp)) return SK_EINVAL;
+      tiles += d.sp.range[0].tiles;
+      sparse = 1;
+    } else {
+      max_ws = std::max(max_ws, ws_len(J.delta, J.n));
+    }
+  }
+  // persistent grid: SMs x resident CTAs; then the zero-skipping jobs' units
+  const size_t smem = (size_t)max_ws * kWsStride +
+                      (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kSpWarp : 0);
+  int grid = 0;
+  cudaError_t e = cudaSuccess;
+  {
+    int dev = 0, sms = 0, nb = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             sp_table_bytes(0) + 8 * kSpWarp +
+                                 ws_len(1, kSparseMinN - 1) * kWsStride);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel, bt, smem);
+    if (e != cudaSuccess) return cuda_status(e);
+    grid = sms * (nb > 0 ? nb : 1);
+  }
+  const int tpu = sp_tiles_per_unit(tiles, (unsigned long long)grid * (bt / 32));
+  unsigned long long chunk = 0;
+  for (int r = 0; r < njobs; ++r) {
+    BatchJobDev& d = hj[r];
+    d.chunk_lo = chunk;
+    if (plan[order[r]].n >= kSparseMinN) {
+      sp_split(&d.sp, tpu);
+      chunk += d.sp.units;
+    } else {
+      chunk += (d.items + 31) / 32;
+    }
   }
   const unsigned long long total_chunks = chunk;
   // device layout: jobs | primes | chunk counter | per-job sums
@@ -325,23 +366,19 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   cudaGraphExec_t exec = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   double kms_last = 0.0, kms_min = 1e300;
-  int grid = 0, launches = 0;
-  cudaError_t e = cudaMalloc(&dbuf, bytes);
+  int launches = 0;
+  e = cudaMalloc(&dbuf, bytes);
   if (e == cudaSuccess) e = cudaHostAlloc(&hbuf, out_bytes, cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaMemcpy(dbuf, hj.data(), sizeof(BatchJobDev) * njobs, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dbuf + off_p, &P, sizeof(Primes), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  const size_t smem = (size_t)max_ws * kWsStride;
-  if (e == cudaSuccess && mode == SK_BATCH_PERSISTENT) {
-    int dev = 0, sms = 0, nb = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel, bt, smem);
-    grid = sms * (nb > 0 ? nb : 1);
+  if (mode == SK_BATCH_PERSISTENT) {
     const unsigned long long need = (total_chunks + bt / 32 - 1) / (bt / 32);
     if ((unsigned long long)grid > need) grid = (int)need;
     launches = 1;
+  } else {
+    grid = 0;
   }
   auto enqueue = [&]() -> cudaError_t {
     cudaError_t r = cudaMemsetAsync(dbuf + off_s, 0, bytes - off_s, s);
@@ -350,12 +387,25 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
       batch_kernel<<<grid, bt, smem, s>>>((const BatchJobDev*)dbuf, njobs, total_chunks,
                                           (const Primes*)(dbuf + off_p), k,
                                           (unsigned long long*)(dbuf + off_s),
-                                          (ExactScratch*)(dbuf + off_j));
+                                          (ExactScratch*)(dbuf + off_j), sparse);
       r = cudaGetLastError();
     } else {
       launches = 0;
       for (int q = 0; q < njobs && r == cudaSuccess; ++q) {
         const JobPlan& J = plan[order[q]];
+        if (J.n >= kSparseMinN) {
+          SpLaunch L;
+          std::memset(&L, 0, sizeof(L));
+          L.job = hj[q].sp;
+          L.P = P;
+          L.nprimes = k;
+          L.scratch = (ExactScratch*)(dbuf + off_j) + q;
+          L.block_threads = bt;
+          L.stream = s;
+          r = sparse_launcher(J.delta, J.n, false)(L);
+          ++launches;
+          continue;
+        }
         ExactLaunch L;
         std::memset(&L, 0, sizeof(L));
         L.job.pres = hj[q].pres;
@@ -424,7 +474,7 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
     rep->prepare_ms = std::chrono::duration<double, std::milli>(t1 - t0).count();
     rep->wall_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     rep->terms = terms;
-    rep->chunks = total_chunks;
+    rep->chunks = item_chunks;
     rep->launches = launches;
     rep->grid = grid;
     rep->block_threads = bt;

@@ -17,6 +17,7 @@
 #include "sk_host_common.h"
 #include "sk_ie.cuh"
 #include "sk_mirror.cuh"
+#include "sk_sparse.cuh"
 
 namespace sk {
 
@@ -107,28 +108,44 @@ ExactLaunchFn ie_launcher(int delta, int n) {
   extern template cudaError_t launch_mirror<0, N>(const ExactLaunch&);              \
   extern template cudaError_t launch_mirror<1, N>(const ExactLaunch&);
 SK_EXTERN_MIRROR(6) SK_EXTERN_MIRROR(7) SK_EXTERN_MIRROR(8) SK_EXTERN_MIRROR(9)
-SK_EXTERN_MIRROR(10) SK_EXTERN_MIRROR(11) SK_EXTERN_MIRROR(12) SK_EXTERN_MIRROR(13)
-SK_EXTERN_MIRROR(14) SK_EXTERN_MIRROR(15) SK_EXTERN_MIRROR(16) SK_EXTERN_MIRROR(17)
-SK_EXTERN_MIRROR(18) SK_EXTERN_MIRROR(19) SK_EXTERN_MIRROR(20) SK_EXTERN_MIRROR(21)
-SK_EXTERN_MIRROR(22) SK_EXTERN_MIRROR(23) SK_EXTERN_MIRROR(24) SK_EXTERN_MIRROR(25)
-SK_EXTERN_MIRROR(26) SK_EXTERN_MIRROR(27) SK_EXTERN_MIRROR(28) SK_EXTERN_MIRROR(29)
-SK_EXTERN_MIRROR(30) SK_EXTERN_MIRROR(31)
+SK_EXTERN_MIRROR(10) SK_EXTERN_MIRROR(11) SK_EXTERN_MIRROR(12)
 #undef SK_EXTERN_MIRROR
 
 #define SK_MROW(N) {launch_mirror<0, N>, launch_mirror<1, N>}
-static const ExactLaunchFn kMirrorTable[kMaxN + 1][2] = {
-    {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr},
-    {nullptr, nullptr}, {nullptr, nullptr},
-    SK_MROW(6), SK_MROW(7), SK_MROW(8), SK_MROW(9), SK_MROW(10), SK_MROW(11), SK_MROW(12),
-    SK_MROW(13), SK_MROW(14), SK_MROW(15), SK_MROW(16), SK_MROW(17), SK_MROW(18), SK_MROW(19),
-    SK_MROW(20), SK_MROW(21), SK_MROW(22), SK_MROW(23), SK_MROW(24), SK_MROW(25), SK_MROW(26),
-    SK_MROW(27), SK_MROW(28), SK_MROW(29), SK_MROW(30), SK_MROW(31)};
+static const ExactLaunchFn kMirrorTable[kSparseMinN - kMirrorMinN][2] = {
+    SK_MROW(6), SK_MROW(7), SK_MROW(8), SK_MROW(9), SK_MROW(10), SK_MROW(11), SK_MROW(12)};
 #undef SK_MROW
-static_assert(kMirrorMinN == 6 && kMaxN == 31, "the table above lists n = 6..31");
+static_assert(kMirrorMinN == 6 && kSparseMinN == 13, "the table above lists n = 6..12");
 
+// Orders from kSparseMinN on walk mirrored items with sparse_launcher.
 ExactLaunchFn mirror_launcher(int delta, int n) {
-  if (delta < 0 || delta > 1 || n < kMirrorMinN || n > kMaxN) return nullptr;
-  return kMirrorTable[n][delta];
+  if (delta < 0 || delta > 1 || n < kMirrorMinN || n >= kSparseMinN) return nullptr;
+  return kMirrorTable[n - kMirrorMinN][delta];
+}
+
+#define SK_EXTERN_SPARSE(N)                                                        \
+  extern template cudaError_t launch_sparse<0, N, 0>(const SpLaunch&);              \
+  extern template cudaError_t launch_sparse<1, N, 0>(const SpLaunch&);              \
+  extern template cudaError_t launch_sparse<0, N, 1>(const SpLaunch&);              \
+  extern template cudaError_t launch_sparse<1, N, 1>(const SpLaunch&);
+SK_EXTERN_SPARSE(13) SK_EXTERN_SPARSE(14) SK_EXTERN_SPARSE(15) SK_EXTERN_SPARSE(16)
+SK_EXTERN_SPARSE(17) SK_EXTERN_SPARSE(18) SK_EXTERN_SPARSE(19) SK_EXTERN_SPARSE(20)
+SK_EXTERN_SPARSE(21) SK_EXTERN_SPARSE(22) SK_EXTERN_SPARSE(23) SK_EXTERN_SPARSE(24)
+SK_EXTERN_SPARSE(25) SK_EXTERN_SPARSE(26) SK_EXTERN_SPARSE(27) SK_EXTERN_SPARSE(28)
+SK_EXTERN_SPARSE(29) SK_EXTERN_SPARSE(30) SK_EXTERN_SPARSE(31)
+#undef SK_EXTERN_SPARSE
+
+#define SK_SROW(N) {{launch_sparse<0, N, 0>, launch_sparse<0, N, 1>}, \
+                    {launch_sparse<1, N, 0>, launch_sparse<1, N, 1>}}
+static const SparseLaunchFn kSparseTable[kMaxN + 1 - kSparseMinN][2][2] = {
+    SK_SROW(13), SK_SROW(14), SK_SROW(15), SK_SROW(16), SK_SROW(17), SK_SROW(18), SK_SROW(19),
+    SK_SROW(20), SK_SROW(21), SK_SROW(22), SK_SROW(23), SK_SROW(24), SK_SROW(25), SK_SROW(26),
+    SK_SROW(27), SK_SROW(28), SK_SROW(29), SK_SROW(30), SK_SROW(31)};
+#undef SK_SROW
+
+SparseLaunchFn sparse_launcher(int delta, int n, bool mirrored) {
+  if (delta < 0 || delta > 1 || n < kSparseMinN || n > kMaxN) return nullptr;
+  return kSparseTable[n - kSparseMinN][delta][mirrored ? 1 : 0];
 }
 
 // Largest walk width of the exact form (compile-time table per (delta, n)).
@@ -181,7 +198,9 @@ struct Plan {
   unsigned long long pres, items;
   uint64_t primes[kMaxPrimes];
   Primes P;
-  ExactLaunchFn fn;
+  ExactLaunchFn fn;        // the dense walk (null for mirrored items of n >= kSparseMinN)
+  SparseLaunchFn sparse;   // the zero-skipping walk (null: none for this plan)
+  bool mirrored;
 };
 
 static int make_plan(int variant, int n, const sk_count_opts* o, Plan* pl,
@@ -310,11 +329,14 @@ static int make_plan(int variant, int n, const sk_count_opts* o, Plan* pl,
   pl->grid = (o && o->grid > 0) ? o->grid : 0;
   const bool mirrored =
       pl->symmetry == SK_SYMMETRY_REVERSAL || pl->symmetry == SK_SYMMETRY_REVERSAL_EVEN;
+  pl->mirrored = mirrored;
+  if (method == kMethodAlgebraic && pl->arith == SK_ARITH_LIMBS)
+    pl->sparse = sparse_launcher(pl->delta, n, mirrored);
   pl->fn = method == kMethodInclusionExclusion     ? ie_launcher(pl->delta, n)
            : mirrored                              ? mirror_launcher(pl->delta, n)
            : pl->arith == SK_ARITH_LIMBS          ? limb_launcher(pl->delta, n)
                                                   : exact_launcher(pl->delta, n, pl->nprimes);
-  if (!pl->fn) return SK_EINVAL;
+  if (!pl->fn && !pl->sparse) return SK_EINVAL;
   return SK_OK;
 }
 
@@ -337,23 +359,39 @@ static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long h
                      int* grid_used) {
   cudaError_t e = cudaMemsetAsync(dscr, 0, sizeof(ExactScratch), st);
   if (e != cudaSuccess) return cuda_status(e);
-  ExactLaunch L;
-  L.job.pres = pl.pres;
-  L.job.items = pl.items;
-  L.job.m = pl.m;
-  L.job.job = 0;
-  L.job.fixed_bit = pl.fixed_bit;
-  L.P = pl.P;
-  L.nprimes = pl.nprimes;
-  L.item_lo = lo;
-  L.item_hi = hi;
-  L.scratch = dscr;
-  L.item_res = item_res;
-  L.block_threads = pl.block_threads;
-  L.grid = pl.grid;
-  L.stream = st;
   cudaEventRecord(e0, st);
-  e = pl.fn(L);
+  // The zero-skipping walk sums whole jobs, aligned power-of-two ranges of
+  // items and mirrored items; it has no sum per item, so item residues and
+  // other ranges take the dense walk.
+  SpLaunch S;
+  if (pl.sparse && !item_res &&
+      (pl.mirrored ? sp_mirror_job(pl.pres, pl.delta, pl.n, pl.m, lo, hi, &S.job)
+                   : sp_plain_job(pl.pres, pl.delta, pl.n, pl.m, pl.fixed_bit, lo, hi, &S.job))) {
+    S.P = pl.P;
+    S.nprimes = pl.nprimes;
+    S.scratch = dscr;
+    S.block_threads = pl.block_threads;
+    S.grid = pl.grid;
+    S.stream = st;
+    e = pl.sparse(S);
+  } else {
+    ExactLaunch L;
+    L.job.pres = pl.pres;
+    L.job.items = pl.items;
+    L.job.m = pl.m;
+    L.job.job = 0;
+    L.job.fixed_bit = pl.fixed_bit;
+    L.P = pl.P;
+    L.nprimes = pl.nprimes;
+    L.item_lo = lo;
+    L.item_hi = hi;
+    L.scratch = dscr;
+    L.item_res = item_res;
+    L.block_threads = pl.block_threads;
+    L.grid = pl.grid;
+    L.stream = st;
+    e = pl.fn ? pl.fn(L) : cudaErrorInvalidValue;
+  }
   if (e != cudaSuccess) return cuda_status(e);
   cudaEventRecord(e1, st);
   ExactScratch h;
