@@ -66,9 +66,9 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
   const int lane = threadIdx.x & 31;
   BatchSmem sm;
   const int warps = blockDim.x >> 5;
-  const int dense = sparse ? sp_table_bytes(0) + warps * kSpWarp : 0;
+  const int dense = sparse ? sp_table_bytes(0) + warps * kBatchWarp : 0;
   sm.tab = (unsigned)__cvta_generic_to_shared(sk_batch_smem);
-  sm.wsm = sm.tab + sp_table_bytes(0) + (threadIdx.x >> 5) * kSpWarp;
+  sm.wsm = sm.tab + sp_table_bytes(0) + (threadIdx.x >> 5) * kBatchWarp;
   sm.ws_col = (signed char*)sk_batch_smem + dense + threadIdx.x;
   if (sparse) sp_build_tables<0>(sk_batch_smem);
   __syncthreads();
@@ -320,7 +320,7 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   }
   // persistent grid: SMs x resident CTAs; then the zero-skipping jobs' units
   const size_t smem = (size_t)max_ws * kWsStride +
-                      (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kSpWarp : 0);
+                      (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kBatchWarp : 0);
   int grid = 0;
   cudaError_t e = cudaSuccess;
   {
@@ -328,7 +328,7 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sp_table_bytes(0) + 8 * kSpWarp +
+                             sp_table_bytes(0) + 8 * kBatchWarp +
                                  ws_len(1, kSparseMinN - 1) * kWsStride);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel, bt, smem);

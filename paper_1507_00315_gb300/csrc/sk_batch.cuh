@@ -24,6 +24,11 @@ struct BatchJobDev {
   int code;                      // delta * 32 + n
 };
 
+// Tiles whose survivors a warp evaluates together, and its shared memory (two
+// CTAs of 8 warps an SM, beside the dense walk's columns).
+constexpr int kBatchGroup = 2;
+constexpr int kBatchWarp = sp_warp_bytes(8, kBatchGroup);
+
 // Shared memory of a CTA as the work functions see it.
 struct BatchSmem {
   signed char* ws_col;           // this thread's column of the dense walk's copy of w
@@ -37,7 +42,7 @@ __device__ __forceinline__ Res4 batch_chunk_impl(const BatchJobDev* job, const P
                                                  const BatchSmem& sm) {
   if constexpr (N >= kSparseMinN) {
     const unsigned long long off = c * (unsigned long long)job->sp.tpu;
-    return sparse_unit<DELTA, N, 0>(&job->sp, off, job->sp.tpu, P, nprimes, sm.tab, sm.wsm);
+    return sparse_unit<DELTA, N, 0, kBatchGroup>(&job->sp, off, job->sp.tpu, P, nprimes, sm.tab, sm.wsm);
   } else {
     const unsigned long long item = c * 32ULL + (threadIdx.x & 31);
     if (item < job->items)

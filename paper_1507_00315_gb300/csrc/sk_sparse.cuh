@@ -25,18 +25,24 @@
 // Zero test.  Term (i, s) has c_d = 0 iff R_d(s) = v_i, v_i = L_d/2 - U_d -
 // H_d(i): a table word [pattern of the partners][v] holds one bit per s.
 // Lane i ORs the words of every even d: the zeros of its 32 terms.
-// Survivors are appended to the warp's list (lane-major, entry = lane, s) and
-// evaluated 32 at a time: two shuffles per word bring a_i and R(s), the bytes
-// are multiplied in int32 groups and the groups in signed radix-2^31 digits
+// Survivors are appended to the warp's list (lane-major, entry = tile, lane, s)
+// and evaluated 32 at a time: a_i comes from shared memory, R(s) by a shuffle
+// per word, the bytes are multiplied in int32 groups and the groups in signed radix-2^31 digits
 // as in sk_exact.cuh, and tail * digit enters 64-bit accumulators (split into
 // 32-bit halves before they can overflow).
 //
-// Bound by instruction issue (82 % of the issue slots, ALU 68 %, multiply pipe
-// 56 % busy, S(17) under ncu): about 1020 warp instructions a tile, 690 of them
-// the survivors' evaluation.  Whole counts against the dense walk (56
-// instructions a term): S(20) 482 and 1086 ms, hooked n = 18 31.4 and 65.0 ms,
-// mirrored L(19) (Lemmas 2.3 + 2.4) 35.1 and 71.5 ms, S(13) 0.12 and 0.10 ms:
-// below n = 13 a lane block clear of the low block's partners does not exist.
+// Group.  The survivors of up to 4 tiles that differ in the fast bits (next to
+// the lane bits, out of the low block's reach: R and the mask rows stay) share
+// one list, so that few evaluations run part empty; the tiles' a rows wait in
+// shared memory, where the 32 entries of an evaluation read few of them.
+//
+// Bound by instruction issue (82 % of the issue slots, ALU 69 %, multiply pipe
+// 60 %, shared-memory pipe 67 % busy, S(17) under ncu): about 945 warp
+// instructions a tile, 600 of them the survivors' evaluation (73 for 32).
+// Whole counts, dense walk (56 instructions a term) and this one: S(20) 1086
+// and 447 ms, hooked n = 18 65.0 and 29.5 ms, mirrored L(19) (Lemmas 2.3 + 2.4)
+// 71.5 and 28.9 ms (one list a tile: 482, 31.4, 35.1 ms).  Below n = 13 no lane
+// block is clear of the low block's partners.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -61,10 +67,16 @@ constexpr int kSpFirst = 256 * 128;
 constexpr int kSpMask = kSpFirst + 2 * 32 * 128;
 __host__ __device__ constexpr int sp_mask_rows(int LB) { return LB ? 72 : 52; }
 __host__ __device__ constexpr int sp_table_bytes(int LB) { return kSpMask + sp_mask_rows(LB) * 256; }
-// Per warp: the survivors' list (at most 1024 two-byte entries), 32 table
-// addresses and 32 bytes of U.
-constexpr int kSpList = 2048;
-constexpr int kSpWarp = kSpList + 128 + 32;
+// Per warp, for groups of TG tiles (bytes): the survivors' list (two-byte
+// entries; at least one tile's 1024, for TG = 4 half as many again as usually
+// survive), the tiles' masks [TG][32], their rows a
+// [TG][32][first 4 words] and [TG][32][other words], 32 table addresses and 32
+// bytes of U.
+__host__ __device__ constexpr int sp_list_cap(int TG) { return TG >= 4 ? 1536 : 1024; }
+__host__ __device__ constexpr int sp_row2(int NQ) { return NQ <= 4 ? 0 : NQ == 5 ? 4 : NQ == 6 ? 8 : 16; }
+__host__ __device__ constexpr int sp_warp_bytes(int NQ, int TG) {
+  return 2 * sp_list_cap(TG) + TG * 32 * (4 + 16 + sp_row2(NQ)) + 128 + 32;
+}
 
 __host__ __device__ inline unsigned sp_popc(unsigned x) {
 #ifdef __CUDA_ARCH__
@@ -367,7 +379,7 @@ __host__ __device__ __forceinline__ void sparse_product(const int (&c)[N],
 // for even d (a sign-extended byte), c_d for odd d (twice the byte plus odd0,
 // -255, or -256 where L_d is even after all: hooked Skolem's d = 1).
 template <int DELTA, int K>
-__host__ __device__ __forceinline__ int sp_factor(unsigned w, int odd0) {
+__host__ __device__ __forceinline__ int sp_factor(unsigned w, int odd0, uint2 unit) {
   constexpr int e = K & 3;
   constexpr int d = 1 + DELTA + K;
 #ifdef __CUDA_ARCH__
@@ -377,7 +389,7 @@ __host__ __device__ __forceinline__ int sp_factor(unsigned w, int odd0) {
     asm("prmt.b32 %0, %1, %1, %2;" : "=r"(v) : "r"(w ^ 0x80808080u), "n"(0x8880 + 0x1111 * e));
     return (int)v;
   } else {
-    return (int)__dp4a(w, 2u << (8 * e), (unsigned)odd0);
+    return (int)__dp4a(w, e < 2 ? unit.x : unit.y, (unsigned)odd0);
   }
 #else
   const int b = (int)((w >> (8 * e)) & 255u);
@@ -387,10 +399,11 @@ __host__ __device__ __forceinline__ int sp_factor(unsigned w, int odd0) {
 
 template <int DELTA, int N, int K = 0>
 __host__ __device__ __forceinline__ void sp_factors(const unsigned (&w)[sp_quads(DELTA, N)],
-                                                   int odd_first, int (&c)[N]) {
+                                                   int odd_first, int odd, uint2 unit,
+                                                   int (&c)[N]) {
   if constexpr (K < N) {
-    c[K] = sp_factor<DELTA, K>(w[K / 4], K == 0 ? odd_first : -255);
-    sp_factors<DELTA, N, K + 1>(w, odd_first, c);
+    c[K] = sp_factor<DELTA, K>(w[K / 4], K == 0 ? odd_first : odd, unit);
+    sp_factors<DELTA, N, K + 1>(w, odd_first, odd, unit, c);
   }
 }
 
@@ -427,7 +440,7 @@ static __device__ __noinline__ void sp_reduce(const long long (&hi)[kMaxDigits],
 
 __device__ __forceinline__ unsigned lds32(unsigned a) {
   unsigned v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
 __device__ __forceinline__ uint4 lds128(unsigned a) {
@@ -451,6 +464,27 @@ __device__ __forceinline__ void sts_u8(unsigned a, unsigned v) {
 }
 __device__ __forceinline__ void sts32(unsigned a, unsigned v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void lds64(unsigned a, unsigned& x, unsigned& y) {
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void sts64(unsigned a, unsigned x, unsigned y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void sts128(unsigned a, unsigned x, unsigned y, unsigned z, unsigned w) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w)
+               : "memory");
+}
+// Takes the highest set bit b of `left` and stores tag | b; nothing where
+// left = 0.
+__device__ __forceinline__ void sp_pop(unsigned& left, unsigned to, unsigned tag) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b32 b, v;\n\t.reg .b16 h;\n\t"
+      "setp.ne.u32 p, %0, 0;\n\tbfind.u32 b, %0;\n\tor.b32 v, b, %2;\n\tcvt.u16.u32 h, v;\n\t"
+      "@p st.shared.u16 [%1], h;\n\tshl.b32 v, 1, b;\n\txor.b32 %0, %0, v;\n\t}"
+      : "+r"(left)
+      : "r"(to), "r"(tag)
+      : "memory");
 }
 // NW (<= 16) words from a 16-byte aligned shared address
 template <int NW>
@@ -486,7 +520,7 @@ __device__ __forceinline__ unsigned sp_disagree(unsigned xl, unsigned xh, int d,
 // Residues of one work unit (tiles tile_lo .. tile_lo + ntiles - 1), this
 // lane's part.  tab, wsm: shared addresses of the CTA's tables and this
 // warp's area.
-template <int DELTA, int N, int LB>
+template <int DELTA, int N, int LB, int TG>
 __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long tile_lo, int ntiles,
                                             const Primes* P, int nprimes, unsigned tab,
                                             unsigned wsm) {
@@ -494,8 +528,11 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
   constexpr DigitPlan dp = make_sparse_plan(DELTA, N);
   constexpr int K = dp.kd;
   constexpr bool kWide = N + DELTA >= 32;
-  static_assert(NQ <= 8 && NT <= 16 && K <= kMaxDigits, "one lane per task");
-  constexpr int kFlush = (1 << dp.max_m) - 32;   // evaluations a tile adds at most: 32
+  static_assert(NQ >= 4 && NQ <= 8 && NT <= 16 && K <= kMaxDigits, "one lane per task");
+  constexpr int kCap = sp_list_cap(TG);
+  // evaluations between flushes: 2^max_m; a batch adds at most kCap / 32
+  constexpr int kFlush = (1 << dp.max_m) - kCap / 32;
+  static_assert(kFlush >= 0, "accumulators hold one batch");
   const SpJob& J = *Jp;
   const int lane = threadIdx.x & 31;
   const unsigned long long pres = J.pres;
@@ -513,8 +550,18 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
   }
   SpTask task = sp_task(DELTA, NQ, NT, LB, lane);
   task.base += tab;
+  // the task's window starts at bit `from` of x, or of x reversed for the lane
+  // block's quads
   const bool hi_stream = lane >= 8 && lane < 16;
+  const int from = task.sh + (hi_stream ? 64 - hb : LB + 5);
+  const bool upper = from >= 32;
   const int odd_first = (sp_popcll(pres & (pres >> 1)) & 1) ? -255 : -256;   // hooked: L_1 even
+  // constants of the odd factors in registers, not rebuilt for every use
+  int odd;
+  uint2 unit;                                    // twice the byte of an odd distance
+  asm volatile("mov.u32 %0, -255;" : "=r"(odd));
+  asm volatile("mov.u32 %0, %1;" : "=r"(unit.x) : "n"(DELTA ? 0x200 : 0x2));
+  asm volatile("mov.u32 %0, %1;" : "=r"(unit.y) : "n"(DELTA ? 0x2000000 : 0x20000));
   // fixed bits above the lane bits: their pairs with the lane bits
   unsigned long long x_fixed = 0;
   if constexpr (LB == 0) x_fixed = sp_tile_bits(J, tile_lo) & ~((1ULL << hb) - 1ULL);
@@ -533,8 +580,9 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
       }
     }
   }
-  const unsigned a_list = wsm, a_addr = wsm + kSpList, a_u = wsm + kSpList + 128;
   const unsigned lane4 = (unsigned)lane * 4u, rlane4 = sp_rev5((unsigned)lane) * 4u;
+  const unsigned a_row = wsm, a_row2 = a_row + TG * 32 * 16, a_mask = a_row2 + TG * 32 * sp_row2(NQ),
+                 a_list = a_mask + TG * 32 * 4, a_addr = a_list + 2 * kCap, a_u = a_addr + 128;
   long long acc[K], alo[K], ahi[K];
 #pragma unroll
   for (int i = 0; i < K; ++i) acc[i] = alo[i] = ahi[i] = 0;
@@ -544,117 +592,176 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
   if constexpr (LB == 1) sh = mirror_shape(N, J.h);
   unsigned r[NQ];
   const unsigned fast_mask = (1u << J.fast) - 1u;
-  for (int tt = 0; tt < ntiles; ++tt) {
-    const unsigned long long T = tile_lo + (unsigned)tt;
+  const unsigned long long fast_step = 1ULL << (hb - J.fast);
+  const int group = J.fast >= 2 ? TG : (TG < (1 << J.fast) ? TG : (1 << J.fast));
+  // 32 list entries from e on: T r_i of each into the accumulators
+  auto evaluate = [&](unsigned e, int sgn) {
+    unsigned w[NQ];
+    const unsigned slot = e >> 6;
+    {
+      const uint4 v = lds128(a_row + slot * 16u);
+      w[0] = v.x;
+      w[1] = v.y;
+      w[2] = v.z;
+      w[3] = v.w;
+    }
+    if constexpr (NQ == 5) {
+      w[4] = lds32(a_row2 + slot * 4u);
+    } else if constexpr (NQ == 6) {
+      lds64(a_row2 + slot * 8u, w[4], w[5]);
+    } else if constexpr (NQ >= 7) {
+      const uint4 v = lds128(a_row2 + slot * 16u);
+      w[4] = v.x;
+      w[5] = v.y;
+      w[6] = v.z;
+      if constexpr (NQ == 8) w[7] = v.w;
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) w[q] -= __shfl_sync(0xffffffffu, r[q], (int)e);
+    int c[N], rd[K], Tl;
+    sp_factors<DELTA, N>(w, odd_first, odd, unit, c);
+    sparse_product<DELTA, N>(c, rd, Tl);
+    Tl *= sgn;
+#pragma unroll
+    for (int i = 0; i < K; ++i) acc[i] = wide_mad_s32(rd[i], Tl, acc[i]);
+  };
+  for (int tt = 0; tt < ntiles; tt += group) {
+    const int here = ntiles - tt < group ? ntiles - tt : group;
+    unsigned tags = 0;                              // sign bit of each tile of the group
+    int cnt = 0;
+    // the group's first pattern; its tiles count up the fast bits
+    const unsigned long long T0 = tile_lo + (unsigned)tt;
     unsigned long long x;
     if constexpr (LB == 0) {
-      x = sp_tile_bits(J, T);
+      x = sp_tile_bits(J, T0);
     } else {
       const int wb = 2 * (J.h - 5);
-      const unsigned long long q = T >> wb;
+      const unsigned long long q = T0 >> wb;
       if (q != q_cur) {
         int weight;
         q_cur = q;
         q_bits = mirror_item_bits(sh, q, &weight);
       }
-      x = q_bits | sp_mirror_walk(J, N, T & ((1ULL << wb) - 1ULL));
+      x = q_bits | sp_mirror_walk(J, N, T0 & ((1ULL << wb) - 1ULL));
     }
-    const unsigned xl = (unsigned)x, xh = (unsigned)(x >> 32);
-    // one distance and one table address per lane
-    const bool fresh = tt == 0 || ((unsigned)T & fast_mask) == 0;   // the low block's rows change
-    if (fresh || hi_stream) {
-      const unsigned long long y = hi_stream ? sp_brevll(x) >> (64 - hb) : x >> (LB + 5);
-      const unsigned win = __funnelshift_r((unsigned)y, (unsigned)(y >> 32), task.sh) & task.msk;
-      unsigned addr = task.base + win * task.mul;
-      if constexpr (LB == 1) addr += (xl & 1u) ? task.x0add : 0u;
-      sts32(a_addr + lane4, addr);
-    }
-    sts_u8(a_u + lane, ubase - sp_disagree<kWide>(xl, xh, du, pml, pmh));
-    __syncwarp();
-    if (fresh) {
-      unsigned al[NQ];
-      lds_words<NQ>(a_addr, al);
+    bool fresh = tt == 0 || ((unsigned)T0 & fast_mask) == 0;        // new rows r
+#pragma unroll 1
+    for (int g = 0; g < here; ++g, x += fast_step, fresh = false) {
+      const unsigned xl = (unsigned)x, xh = (unsigned)(x >> 32);
+      // one distance and one table address per lane
+      {
+        const unsigned zl = hi_stream ? __brev(xh) : xl, zh = hi_stream ? __brev(xl) : xh;
+        const unsigned win =
+            __funnelshift_r(upper ? zh : zl, upper ? 0u : zh, (unsigned)from) & task.msk;
+        unsigned addr = task.base + win * task.mul;
+        if constexpr (LB == 1) addr += (xl & 1u) ? task.x0add : 0u;
+        sts32(a_addr + lane4, addr);
+      }
+      sts_u8(a_u + lane, ubase - sp_disagree<kWide>(xl, xh, du, pml, pmh));
+      tags |= (((unsigned)__popc(xl ^ xh ^ (unsigned)g)) & 1u) << g;
+      __syncwarp();
+      if (fresh) {
+        unsigned al[NQ];
+        lds_words<NQ>(a_addr, al);
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) r[q] = lds32(al[q] + lane4);
-      if constexpr (LB == 1) {
-        // bit 0 pairs with low bit j at distance 1 + j
+        for (int q = 0; q < NQ; ++q) r[q] = lds32(al[q] + lane4);
+        if constexpr (LB == 1) {
+          // bit 0 pairs with low bit j at distance 1 + j
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-          const int k = 1 + j - D0;
-          if (k >= 0 && k < N) r[k / 4] += (((unsigned)(lane >> j) ^ xl) & 1u) << (8 * (k & 3));
+          for (int j = 0; j < 5; ++j) {
+            const int k = 1 + j - D0;
+            if (k >= 0 && k < N) r[k / 4] += (((unsigned)(lane >> j) ^ xl) & 1u) << (8 * (k & 3));
+          }
         }
       }
-    }
-    unsigned a[NQ];
-    {
-      unsigned ah[NQ], u[NQ];
-      lds_words<NQ>(a_addr + 32, ah);
-      lds_words<NQ>(a_u, u);
+      unsigned a[NQ];
+      {
+        unsigned ah[NQ], u[NQ];
+        lds_words<NQ>(a_addr + 32, ah);
+        lds_words<NQ>(a_u, u);
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) a[q] = u[q] - lds32(ah[q] + rlane4) - st[q];
-    }
-    // zeros of this lane's 32 terms
-    unsigned zero = 0;
-    {
-      unsigned am[NT];
-      lds_words<NT>(a_addr + 64, am);
-#pragma unroll
-      for (int i = 0; i < NT; ++i) {
-        const int k = 2 + 2 * i - D0;             // d = 2 + 2 i
-        zero |= lds32(__dp4a(a[k / 4], 4u << (8 * (k & 3)), am[i]));
+        for (int q = 0; q < NQ; ++q) a[q] = u[q] - lds32(ah[q] + rlane4) - st[q];
       }
-    }
-    unsigned left = ~zero;
-    // append the survivors: lane-major, entry = parity of the tile, lane, s
-    const int cnt = __popc(left);
-    int incl = cnt;
+      const unsigned slot = (unsigned)(g * 32 + lane);
+      sts128(a_row + slot * 16u, a[0], a[1], a[2], a[3]);
+      if constexpr (NQ == 5) sts32(a_row2 + slot * 4u, a[4]);
+      if constexpr (NQ == 6) sts64(a_row2 + slot * 8u, a[4], a[5]);
+      if constexpr (NQ >= 7) sts128(a_row2 + slot * 16u, a[4], a[5], a[6], NQ == 8 ? a[NQ - 1] : 0u);
+      // zeros of this lane's 32 terms
+      unsigned zero = 0;
+      {
+        unsigned am[NT];
+        lds_words<NT>(a_addr + 64, am);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned at = a_list + 2u * (unsigned)(incl - cnt);
-    const unsigned tag = (((unsigned)__popc(xl ^ xh) & 1u) << 10) | ((unsigned)lane << 5);
-    const int most = __reduce_max_sync(0xffffffffu, cnt);
-    for (int j = 0; j < most; j += 4) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        unsigned b, bit;                          // highest set bit; none: b = ~0, bit = 0
-        asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(left));
-        asm("shl.b32 %0, 1, %1;" : "=r"(bit) : "r"(b));
-        if (left) sts_u16(at + 2 * i, tag | b);
-        left ^= bit;
+        for (int i = 0; i < NT; ++i) {
+          const int k = 2 + 2 * i - D0;             // d = 2 + 2 i
+          zero |= lds32(__dp4a(a[k / 4], 4u << (8 * (k & 3)), am[i]));
+        }
       }
-      at += 8;
+      sts32(a_mask + (unsigned)g * 128u + lane4, ~zero);
+      cnt += __popc(~zero);
+      __syncwarp();                                 // before the next tile's addresses
     }
-    __syncwarp();
-    // evaluate them, 32 at a time
-    for (int i0 = 0; i0 < total; i0 += 32) {
-      const unsigned e = lds_u16(a_list + 2u * (unsigned)(i0 + lane));
-      const int sgn = i0 + lane < total ? 1 - 2 * (int)(__popc(e) & 1u) : 0;
-      unsigned w[NQ];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q)
-        w[q] = __shfl_sync(0xffffffffu, a[q], (int)(e >> 5)) - __shfl_sync(0xffffffffu, r[q], (int)e);
-      int c[N], rd[K], Tl;
-      sp_factors<DELTA, N>(w, odd_first, c);
-      sparse_product<DELTA, N>(c, rd, Tl);
-      Tl *= sgn;
-#pragma unroll
-      for (int i = 0; i < K; ++i) acc[i] = wide_mad_s32(rd[i], Tl, acc[i]);
-    }
-    evals += (total + 31) >> 5;
-    if (evals > kFlush) {
-      evals = 0;
-#pragma unroll
-      for (int i = 0; i < K; ++i) {
-        alo[i] += (long long)(unsigned)acc[i];
-        ahi[i] += acc[i] >> 32;
-        acc[i] = 0;
+    // the group's survivors in one batch, or, if the list could not hold
+    // them, tile by tile
+    // (sums by warp reduction: uniform, so the loops below are too)
+    int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
+    const bool whole = total <= kCap;
+    for (int g0 = 0; g0 < here;) {
+      const int g1 = whole ? here : g0 + 1;
+      if (!whole) {
+        cnt = __popc(lds32(a_mask + (unsigned)g0 * 128u + lane4));
+        total = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
       }
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      // lane-major; entry = tile, lane, sign of tile, s
+      unsigned at = a_list + 2u * (unsigned)(incl - cnt);
+      for (int g = g0; g < g1; ++g) {
+        unsigned left = lds32(a_mask + (unsigned)g * 128u + lane4);
+        const unsigned tag = ((unsigned)(g * 32 + lane) << 6) | (((tags >> g) & 1u) << 5);
+        const int mine = __popc(left), most = __reduce_max_sync(0xffffffffu, mine);
+        unsigned to = at;
+        for (int j = 0; j < most; j += 2) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            sp_pop(left, to + 2 * i, tag);
+          }
+          to += 4;
+        }
+        at += 2u * (unsigned)mine;
+      }
+      __syncwarp();
+      // (the next entry is fetched ahead; past the end it reads the addresses
+      // that follow the list, unused)
+      int i0 = 0;
+      unsigned e = lds_u16(a_list + 2u * (unsigned)lane);
+      for (; i0 + 32 <= total; i0 += 32) {
+        const unsigned en = lds_u16(a_list + 2u * (unsigned)(i0 + 32 + lane));
+        evaluate(e, 1 - 2 * (int)(__popc(e) & 1u));
+        e = en;
+      }
+      if (i0 < total) {
+        const bool in = i0 + lane < total;
+        evaluate(in ? e : 0u, in ? 1 - 2 * (int)(__popc(e) & 1u) : 0);
+      }
+      evals += (total + 31) >> 5;
+      if (evals > kFlush) {
+        evals = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+          alo[i] += (long long)(unsigned)acc[i];
+          ahi[i] += acc[i] >> 32;
+          acc[i] = 0;
+        }
+      }
+      __syncwarp();
+      g0 = g1;
     }
-    __syncwarp();
   }
   long long h6[kMaxDigits] = {}, l6[kMaxDigits] = {};
 #pragma unroll
@@ -669,10 +776,15 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
 
 // ------------------------------------------------------------ kernel
 
-// Three CTAs of 8 warps an SM (80 registers a thread; 72 KB of tables and
-// lists each): S(18) in 32.6 ms, with two (128 registers) 35.3 ms.
+// One CTA an SM: 24 warps (80 registers a thread), 16 where the rows of the
+// largest orders would not fit beside the tables.
+constexpr int kSpGroup = 4;
+__host__ __device__ constexpr int sp_max_warps(int DELTA, int N) {
+  return sp_quads(DELTA, N) <= 6 ? 24 : 16;
+}
+
 template <int DELTA, int N, int LB>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(32 * sp_max_warps(DELTA, N), 1)
     sparse_kernel(SpJob J, Primes P, int nprimes, ExactScratch* scr) {
   extern __shared__ __align__(16) unsigned char sp_smem[];
   __shared__ SpJob sJ;
@@ -685,12 +797,15 @@ __global__ void __launch_bounds__(256, 3)
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const unsigned tab = (unsigned)__cvta_generic_to_shared(sp_smem);
-  const unsigned wsm = tab + sp_table_bytes(LB) + (threadIdx.x >> 5) * kSpWarp;
+  const unsigned wsm =
+      tab + sp_table_bytes(LB) + (threadIdx.x >> 5) * sp_warp_bytes(sp_quads(DELTA, N), kSpGroup);
   unsigned long long tot[kMaxPrimes] = {0, 0, 0, 0};
   for (;;) {
     unsigned long long u = 0;
     if (lane == 0) u = atomicAdd(&scr->counter, 1ULL);
-    u = __shfl_sync(0xffffffffu, u, 0);
+    // lane 0's unit, by warp reduction: uniform registers hold it from here on
+    u = ((unsigned long long)__reduce_max_sync(0xffffffffu, (unsigned)(u >> 32)) << 32) |
+        __reduce_max_sync(0xffffffffu, lane == 0 ? (unsigned)u : 0u);
     if (u >= sJ.units) break;
     int g = 0;
     while (g + 1 < sJ.nrange && u >= sJ.range[g + 1].unit_lo) ++g;
@@ -698,7 +813,8 @@ __global__ void __launch_bounds__(256, 3)
     const unsigned long long off = (u - R.unit_lo) * (unsigned long long)sJ.tpu;
     const unsigned long long rest = R.tiles - off;
     const int nt = rest < (unsigned long long)sJ.tpu ? (int)rest : sJ.tpu;
-    const Res4 r = sparse_unit<DELTA, N, LB>(&sJ, R.tile_lo + off, nt, &sP, nprimes, tab, wsm);
+    const Res4 r =
+        sparse_unit<DELTA, N, LB, kSpGroup>(&sJ, R.tile_lo + off, nt, &sP, nprimes, tab, wsm);
 #pragma unroll
     for (int i = 0; i < kMaxPrimes; ++i) {
       if (i >= nprimes) break;
@@ -824,7 +940,11 @@ cudaError_t launch_sparse(const SpLaunch& L) {
   const int bt = L.block_threads;
   if (L.nprimes < 1 || L.nprimes > kMaxPrimes || bt < 32 || bt > 256 || (bt & 31))
     return cudaErrorInvalidValue;
-  const size_t smem = sp_table_bytes(LB) + (size_t)(bt / 32) * kSpWarp;
+  // 256 threads (the default) stand for the widest CTA of this walk
+  constexpr int kWarps = sp_max_warps(DELTA, N);
+  constexpr int kArea = sp_warp_bytes(sp_quads(DELTA, N), kSpGroup);
+  const int warps = bt == 256 ? kWarps : bt / 32;
+  const size_t smem = sp_table_bytes(LB) + (size_t)warps * kArea;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -832,9 +952,10 @@ cudaError_t launch_sparse(const SpLaunch& L) {
   int nb = keyed ? occ.per_sm[dev][bt / 32].load(std::memory_order_relaxed) : 0;
   if (nb <= 0) {                  // first launch of this shape on the device
     e = cudaFuncSetAttribute(sparse_kernel<DELTA, N, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sp_table_bytes(LB) + 8 * kSpWarp);
+                             sp_table_bytes(LB) + kWarps * kArea);
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sparse_kernel<DELTA, N, LB>, bt, smem);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sparse_kernel<DELTA, N, LB>,
+                                                        32 * warps, smem);
     if (e != cudaSuccess) return e;
     if (nb <= 0) nb = 1;
     if (keyed) occ.per_sm[dev][bt / 32].store(nb, std::memory_order_relaxed);
@@ -843,13 +964,14 @@ cudaError_t launch_sparse(const SpLaunch& L) {
   SpJob J = L.job;
   unsigned long long tiles = 0;
   for (int g = 0; g < J.nrange; ++g) tiles += J.range[g].tiles;
-  sp_split(&J, sp_tiles_per_unit(tiles, wave * (bt / 32)));
+  sp_split(&J, sp_tiles_per_unit(tiles, wave * warps));
   unsigned long long grid = L.grid > 0 ? (unsigned long long)L.grid : wave;
   if (L.grid <= 0) {
-    const unsigned long long need = (J.units + bt / 32 - 1) / (bt / 32);
+    const unsigned long long need = (J.units + warps - 1) / warps;
     if (grid > need) grid = need;
   }
-  sparse_kernel<DELTA, N, LB><<<(unsigned)grid, bt, smem, L.stream>>>(J, L.P, L.nprimes, L.scratch);
+  sparse_kernel<DELTA, N, LB>
+      <<<(unsigned)grid, 32 * warps, smem, L.stream>>>(J, L.P, L.nprimes, L.scratch);
   return cudaGetLastError();
 }
 

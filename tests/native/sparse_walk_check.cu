@@ -128,7 +128,7 @@ static int check_tiles(const SpJob& J, std::mt19937_64& rng, int samples) {
             if (k >= 0) w[k / 4] -= (unsigned)((x & 1) ^ ((s >> j) & 1)) << (8 * (k & 3));
           }
         int c[N];
-        sp_factors<D, N>(w, odd_first, c);
+        sp_factors<D, N>(w, odd_first, -255, make_uint2(0, 0), c);
         const u64 full = x | ((u64)s << LB) | ((u64)i << hb);
         bool none = true;
         for (int k = 0; k < N; ++k) {
