@@ -65,6 +65,8 @@ struct ExactJob {
   unsigned long long items;  // number of work items (2^{F-m}, F free bits)
   int m;                     // walk bits per item
   int job;                   // slot index of this job's residues
+  int split;                 // 2^split adjacent items of this launch report one
+                             // residue (item_res only; at most 5)
   int fixed_bit;             // 0: none; else a free bit >= m held at +1 (Lemma
                              // 2.4): item indices skip it
 };

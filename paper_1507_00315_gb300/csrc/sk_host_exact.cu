@@ -377,14 +377,22 @@ static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long h
   } else {
     ExactLaunch L;
     L.job.pres = pl.pres;
-    L.job.items = pl.items;
-    L.job.m = pl.m;
+    // few items: narrower ones (mirrored items keep their shape)
+    int dev = 0;
+    e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_status(e);
+    const int split = pl.mirrored ? 0
+                      : item_res  ? item_split(hi - lo, pl.m, pl.U + 3, 5, device_sm_count(dev))
+                                  : item_split(hi - lo, pl.m, pl.U + 1, pl.m, device_sm_count(dev));
+    L.job.items = pl.items << split;
+    L.job.m = pl.m - split;
     L.job.job = 0;
+    L.job.split = split;
     L.job.fixed_bit = pl.fixed_bit;
     L.P = pl.P;
     L.nprimes = pl.nprimes;
-    L.item_lo = lo;
-    L.item_hi = hi;
+    L.item_lo = lo << split;
+    L.item_hi = hi << split;
     L.scratch = dscr;
     L.item_res = item_res;
     L.block_threads = pl.block_threads;

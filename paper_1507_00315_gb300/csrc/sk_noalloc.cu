@@ -100,14 +100,19 @@ extern "C" int skolem_item_residues_noalloc(int variant, int n, int m, uint64_t 
   if (e != cudaSuccess) return cuda_status(e);
   ExactLaunch L;
   L.job.pres = position_mask(variant, n);
-  L.job.items = items;
-  L.job.m = m;
+  int dev = 0;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_status(e);
+  const int split = item_split(count, m, U + 3, 5, device_sm_count(dev));
+  L.job.items = items << split;
+  L.job.m = m - split;
   L.job.job = 0;
+  L.job.split = split;
   L.job.fixed_bit = 0;
   L.P = P;
   L.nprimes = k;
-  L.item_lo = q_lo;
-  L.item_hi = q_lo + count;
+  L.item_lo = q_lo << split;
+  L.item_hi = (q_lo + count) << split;
   L.scratch = rec;
   L.item_res = item_res;
   L.block_threads = 256;
