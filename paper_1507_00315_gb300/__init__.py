@@ -259,6 +259,11 @@ def _variant(v) -> int:
     return int(v)
 
 
+def _rows(flat, k: int):
+    """A ctypes array of rows of k words as a list of lists of ints."""
+    return _np().ctypeslib.as_array(flat).reshape(-1, k).tolist()
+
+
 def default_primes():
     out = (ctypes.c_uint64 * 4)()
     lib().sk_default_primes(out)
@@ -346,7 +351,7 @@ def extended_item_residues(n: int, hole: int, m: int, q_lo: int, count_: int, pr
     st = lib().sk_extended_item_residues(n, hole, m, q_lo, count_, k, P, out)
     if st != SK_OK:
         raise SkolemError(st, "sk_extended_item_residues")
-    return [list(out[i * k:(i + 1) * k]) for i in range(count_)]
+    return _rows(out, k)
 
 
 def ie_item_residues(variant, n: int, m: int, q_lo: int, count_: int, primes):
@@ -357,7 +362,7 @@ def ie_item_residues(variant, n: int, m: int, q_lo: int, count_: int, primes):
     st = lib().sk_ie_item_residues(_variant(variant), n, m, q_lo, count_, k, P, out)
     if st != SK_OK:
         raise SkolemError(st, "sk_ie_item_residues")
-    return [list(out[i * k:(i + 1) * k]) for i in range(count_)]
+    return _rows(out, k)
 
 
 def count_plan(variant, n: int, **kw):
@@ -389,7 +394,7 @@ def item_residues(variant, n: int, m: int, q_lo: int, count_: int, primes, arith
     st = lib().skolem_item_residues_ex(_variant(variant), n, m, q_lo, count_, k, P, arith, out)
     if st != SK_OK:
         raise SkolemError(st, "skolem_item_residues")
-    return [list(out[i * k:(i + 1) * k]) for i in range(count_)]
+    return _rows(out, k)
 
 
 def count_from_residues(variant, n: int, residues, primes=None,
@@ -424,7 +429,7 @@ def item_residues_noalloc(variant, n: int, m: int, q_lo: int, count_: int, prime
     st = lib().skolem_item_residues_noalloc(_variant(variant), n, m, q_lo, count_, k, P, stream, out)
     if st != SK_OK:
         raise SkolemError(st, "skolem_item_residues_noalloc")
-    return [list(out[i * k:(i + 1) * k]) for i in range(count_)]
+    return _rows(out, k)
 
 
 def _batch_opts(nprimes=0, primes=None, convention=REFLECTIONS_IDENTIFIED, mode=BATCH_PERSISTENT,

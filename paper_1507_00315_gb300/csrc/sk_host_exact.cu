@@ -17,6 +17,7 @@
 #include "sk_host_common.h"
 #include "sk_ie.cuh"
 #include "sk_mirror.cuh"
+#include "sk_pool.h"
 #include "sk_sparse.cuh"
 
 namespace sk {
@@ -352,14 +353,22 @@ static void unmont(const Plan& pl, uint64_t* res) {
   }
 }
 
+// The launch record's place in a call's memory.
+constexpr size_t kRecordBytes = 256;
+static_assert(sizeof(ExactScratch) <= kRecordBytes, "launch record");
+
 // One launch over items [lo, hi): raw residues into res (host).
-static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long hi,
-                     ExactScratch* dscr, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1,
-                     uint64_t* res, double* kernel_ms, unsigned long long* item_res,
-                     int* grid_used) {
+// With item_bytes, the items' residues too: in the call's memory (device and
+// pinned host) after the launch record.
+static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long hi, CallScope& cs,
+                     uint64_t* res, double* kernel_ms, size_t item_bytes = 0) {
+  const cudaStream_t st = cs.stream();
+  ExactScratch* dscr = (ExactScratch*)cs.dmem();
+  unsigned long long* item_res =
+      item_bytes ? (unsigned long long*)(cs.dmem() + kRecordBytes) : nullptr;
   cudaError_t e = cudaMemsetAsync(dscr, 0, sizeof(ExactScratch), st);
   if (e != cudaSuccess) return cuda_status(e);
-  cudaEventRecord(e0, st);
+  cudaEventRecord(cs.e0(), st);
   // The zero-skipping walk sums whole jobs, aligned power-of-two ranges of
   // items and mirrored items; it has no sum per item, so item residues and
   // other ranges take the dense walk.
@@ -401,17 +410,17 @@ static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long h
     e = pl.fn ? pl.fn(L) : cudaErrorInvalidValue;
   }
   if (e != cudaSuccess) return cuda_status(e);
-  cudaEventRecord(e1, st);
-  ExactScratch h;
-  e = cudaMemcpyAsync(&h, dscr, sizeof(h), cudaMemcpyDeviceToHost, st);
+  cudaEventRecord(cs.e1(), st);
+  e = cudaMemcpyAsync(cs.hmem(), dscr, item_bytes ? kRecordBytes + item_bytes : sizeof(ExactScratch),
+                      cudaMemcpyDeviceToHost, st);
   if (e != cudaSuccess) return cuda_status(e);
-  e = cudaStreamSynchronize(st);
+  e = cs.drain();
   if (e != cudaSuccess) return cuda_status(e);
   float ms = 0.f;
-  cudaEventElapsedTime(&ms, e0, e1);
+  cudaEventElapsedTime(&ms, cs.e0(), cs.e1());
   *kernel_ms += ms;
+  const ExactScratch& h = *(const ExactScratch*)cs.hmem();
   for (int i = 0; i < pl.nprimes; ++i) res[i] = scratch_residue(h, i, pl.primes[i]);
-  if (grid_used) *grid_used = pl.grid;
   return SK_OK;
 }
 
@@ -636,12 +645,6 @@ int count_impl(int variant, int n, const sk_count_opts* o, sk_u128* out, sk_coun
     if (out) *out = sk_u128{0, 0};
     return SK_OK;
   }
-  cudaStream_t stream = (o && o->stream) ? (cudaStream_t)o->stream : nullptr;
-  bool own_stream = false;
-  if (!stream) {
-    if (cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) != cudaSuccess) return SK_ECUDA;
-    own_stream = true;
-  }
   const bool ckpt_on = o && o->checkpoint_path && o->checkpoint_path[0];
   const unsigned long long chunk = plan_chunk_items(pl, o, ckpt_on);
   const unsigned long long nchunks = (pl.items + chunk - 1) / chunk;
@@ -654,7 +657,7 @@ int count_impl(int variant, int n, const sk_count_opts* o, sk_u128* out, sk_coun
     ck.path = o->checkpoint_path;
     ck.header = ckpt_header(pl, chunk, nchunks);
     st = ckpt_load(&ck, pl);
-    if (st) { if (own_stream) cudaStreamDestroy(stream); return st; }
+    if (st) return st;
     FILE* f = std::fopen(ck.path.c_str(), "rb");
     if (f) {
       std::fseek(f, 0, SEEK_END);
@@ -664,12 +667,8 @@ int count_impl(int variant, int n, const sk_count_opts* o, sk_u128* out, sk_coun
     for (auto h : ck.have) resumed += h;
   }
 
-  ExactScratch* dscr = nullptr;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  cudaError_t ce = cudaMalloc(&dscr, sizeof(ExactScratch));
-  if (ce != cudaSuccess) { if (own_stream) cudaStreamDestroy(stream); return cuda_status(ce); }
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
+  CallScope cs(kRecordBytes, kRecordBytes, o ? o->stream : nullptr);
+  if (cs.error() != cudaSuccess) return cuda_status(cs.error());
   uint64_t H[kMaxPrimes] = {0, 0, 0, 0};
   double kms = 0.0;
   uint64_t done_new = 0, done_total = resumed;
@@ -681,7 +680,7 @@ int count_impl(int variant, int n, const sk_count_opts* o, sk_u128* out, sk_coun
     } else {
       if (max_new && done_new >= max_new) continue;
       unsigned long long lo = c * chunk, hi = lo + chunk < pl.items ? lo + chunk : pl.items;
-      st = run_chunk(pl, lo, hi, dscr, stream, e0, e1, r, &kms, nullptr, nullptr);
+      st = run_chunk(pl, lo, hi, cs, r, &kms);
       if (st) break;
       if (ckpt_on) {
         st = ckpt_append(ck, !file_exists, c, r, pl.nprimes);
@@ -694,10 +693,6 @@ int count_impl(int variant, int n, const sk_count_opts* o, sk_u128* out, sk_coun
     }
     for (int i = 0; i < pl.nprimes; ++i) H[i] = (H[i] + r[i]) % pl.primes[i];
   }
-  cudaFree(dscr);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  if (own_stream) cudaStreamDestroy(stream);
   if (st) return st;
   const bool complete = done_total == nchunks;
   unmont(pl, H);
@@ -763,34 +758,14 @@ int item_residues_impl(int variant, int n, int m, uint64_t q_lo, uint64_t count,
   if (q_lo >= pl.items || count > pl.items - q_lo) return SK_EINVAL;
   st = check_device();
   if (st) return st;
-  cudaStream_t stream;
-  if (cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) != cudaSuccess) return SK_ECUDA;
-  ExactScratch* dscr = nullptr;
-  unsigned long long* dres = nullptr;
-  cudaError_t ce = cudaMalloc(&dscr, sizeof(ExactScratch));
-  if (ce == cudaSuccess) ce = cudaMalloc(&dres, count * pl.nprimes * sizeof(unsigned long long));
-  if (ce != cudaSuccess) {
-    cudaFree(dscr);
-    cudaStreamDestroy(stream);
-    return cuda_status(ce);
-  }
-  cudaEvent_t e0, e1;
-  cudaEventCreate(&e0);
-  cudaEventCreate(&e1);
+  const size_t bytes = count * pl.nprimes * sizeof(uint64_t);
+  CallScope cs(kRecordBytes + bytes, kRecordBytes + bytes, nullptr);
+  if (cs.error() != cudaSuccess) return cuda_status(cs.error());
   uint64_t r[kMaxPrimes];
   double kms = 0;
-  st = run_chunk(pl, q_lo, q_lo + count, dscr, stream, e0, e1, r, &kms, dres, nullptr);
-  std::vector<uint64_t> h(count * pl.nprimes);
-  if (!st) {
-    ce = cudaMemcpy(h.data(), dres, h.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost);
-    if (ce != cudaSuccess) st = cuda_status(ce);
-  }
-  cudaFree(dscr);
-  cudaFree(dres);
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  cudaStreamDestroy(stream);
+  st = run_chunk(pl, q_lo, q_lo + count, cs, r, &kms, bytes);
   if (st) return st;
+  uint64_t* h = (uint64_t*)(cs.hmem() + kRecordBytes);
   for (uint64_t q = 0; q < count; ++q) {
     unmont(pl, &h[q * pl.nprimes]);
     for (int i = 0; i < pl.nprimes; ++i) out[q * pl.nprimes + i] = h[q * pl.nprimes + i];

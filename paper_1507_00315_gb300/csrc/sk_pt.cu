@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "sk_host_common.h"
+#include "sk_pool.h"
 #include "sk_pt.cuh"
 
 namespace sk {
@@ -319,18 +320,17 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   p.groups = groups;
   const size_t n_hist = (size_t)groups * M * nb, n_fin = final_slots ? (size_t)L * M * n : 0;
   const size_t bytes = (tm.size() + ts.size() + n_hist + 2 * (size_t)M + 1) * 8 + n_fin;
-  cudaStream_t s = (cudaStream_t)stream;
-  bool own = false;
-  if (!s) {
-    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return SK_ECUDA;
-    own = true;
-  }
-  unsigned long long* d = nullptr;
-  cudaError_t e = cudaMalloc(&d, bytes);
-  if (e != cudaSuccess) {
-    if (own) cudaStreamDestroy(s);
-    return cuda_status(e);
-  }
+  // the call's stream, events, device memory and pinned host memory (the
+  // thresholds on the way in, the counts on the way out)
+  const size_t n_out = n_hist + 2 * (size_t)M + 1, n_thr = tm.size() + ts.size();
+  CallScope cs(bytes, (n_thr + n_out) * 8, stream);
+  if (cs.error() != cudaSuccess) return cuda_status(cs.error());
+  const cudaStream_t s = cs.stream();
+  unsigned long long* d = (unsigned long long*)cs.dmem();
+  unsigned long long* hthr = (unsigned long long*)cs.hmem();
+  unsigned long long* hh = hthr + n_thr;
+  std::copy(tm.begin(), tm.end(), hthr);
+  std::copy(ts.begin(), ts.end(), hthr + tm.size());
   unsigned long long* dtm = d;
   unsigned long long* dts = dtm + tm.size();
   unsigned long long* dh = dts + ts.size();
@@ -338,10 +338,8 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   unsigned long long* das = dam + M;
   unsigned long long* dtrips = das + M;
   unsigned char* dfin = final_slots ? (unsigned char*)(dtrips + 1) : nullptr;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  e = cudaMemcpyAsync(dtm, tm.data(), tm.size() * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dts, ts.data(), ts.size() * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dh, 0, (n_hist + 2 * (size_t)M + 1) * 8, s);
+  cudaError_t e = cudaMemcpyAsync(dtm, hthr, n_thr * 8, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dh, 0, n_out * 8, s);
   const size_t smem = pt_smem_bytes(n, W, p.warps_per_block);
   const bool trips = round_trips != nullptr;
   const auto kernel = W == 2 ? (trips ? pt_kernel<2, true> : pt_kernel<2, false>)
@@ -357,25 +355,18 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   const int lpb = p.warps_per_block / W;
   const int need = (L + lpb - 1) / lpb;
   if (grid > need) grid = need;
-  if (e == cudaSuccess) e = cudaEventCreate(&e0);
-  if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  if (e == cudaSuccess) e = cudaEventRecord(e0, s);
+  if (e == cudaSuccess) e = cudaEventRecord(cs.e0(), s);
   if (e == cudaSuccess) {
     kernel<<<grid, 32 * p.warps_per_block, smem, s>>>(p, dtm, dts, dh, dam, das, dfin, dtrips);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaEventRecord(e1, s);
-  std::vector<unsigned long long> hh(n_hist + 2 * (size_t)M + 1);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hh.data(), dh, hh.size() * 8, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaEventRecord(cs.e1(), s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hh, dh, n_out * 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && final_slots)
     e = cudaMemcpyAsync(final_slots, dfin, n_fin, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = cs.drain();
   float ms = 0.f;
-  if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-  if (e0) cudaEventDestroy(e0);
-  if (e1) cudaEventDestroy(e1);
-  cudaFree(d);
-  if (own) cudaStreamDestroy(s);
+  if (e == cudaSuccess) cudaEventElapsedTime(&ms, cs.e0(), cs.e1());
   if (e != cudaSuccess) return cuda_status(e);
   const size_t per = (size_t)M * nb;
   for (size_t i = 0; i < per; ++i) {
@@ -394,20 +385,41 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   return SK_OK;
 }
 
+namespace {
+
+// What the estimator needs beside the histograms: e^{-(beta_{j+1} - beta_j) E}
+// for every rung but the last, and log(1/2 Z(0)).  Once per ladder: these
+// exponentials, in software where long double has 113 bits, took 10 ms of an
+// estimate when each of its 16 groups computed them again.
+struct PtWeights {
+  std::vector<long double> w;               // [M - 1][2n+1]
+  long double logs;
+};
+
+PtWeights pt_weights(int variant, int n, int M, const double* beta) {
+  const int nb = 2 * n + 1, delta = variant == SK_LANGFORD ? 1 : 0;
+  PtWeights p;
+  p.logs = std::log(0.5L);
+  for (int k = 1; k <= n; ++k) p.logs += std::log((long double)(2 * n - (k + delta)));
+  p.w.resize((size_t)(M > 1 ? M - 1 : 0) * nb);
+  for (int j = 0; j + 1 < M; ++j)
+    for (int E = 0; E < nb; ++E)
+      p.w[(size_t)j * nb + E] = std::exp(-(long double)(beta[j + 1] - beta[j]) * E);
+  return p;
+}
+
 // Sec. 3: S ~ 1/2 Z(0) prod_j Ratio(j); Ratio(j) = mean of
 // e^{-(beta_{j+1} - beta_j) E} at rung j, and for the last rung
 // (beta_{M+1} = infinity) the fraction of samples with E = 0.
-double pt_estimate_from_hist(int variant, int n, int M, const double* beta, const uint64_t* hist,
-                             double* ratios) {
-  const int nb = 2 * n + 1, delta = variant == SK_LANGFORD ? 1 : 0;
-  long double logs = std::log(0.5L);
-  for (int k = 1; k <= n; ++k) logs += std::log((long double)(2 * n - (k + delta)));
+double estimate_with(const PtWeights& p, int n, int M, const uint64_t* hist, double* ratios) {
+  const int nb = 2 * n + 1;
+  long double logs = p.logs;
   for (int j = 0; j < M; ++j) {
     long double tot = 0, acc = 0;
     for (int E = 0; E < nb; ++E) {
       const long double h = (long double)hist[j * nb + E];
       tot += h;
-      if (j + 1 < M) acc += h * std::exp(-(long double)(beta[j + 1] - beta[j]) * E);
+      if (j + 1 < M) acc += h * p.w[(size_t)j * nb + E];
       else if (E == 0) acc += h;
     }
     const long double rr = tot > 0 ? acc / tot : 0;
@@ -417,6 +429,13 @@ double pt_estimate_from_hist(int variant, int n, int M, const double* beta, cons
   return (double)std::exp(logs);
 }
 
+}  // namespace
+
+double pt_estimate_from_hist(int variant, int n, int M, const double* beta, const uint64_t* hist,
+                             double* ratios) {
+  return estimate_with(pt_weights(variant, n, M, beta), n, M, hist, ratios);
+}
+
 // Pooled estimate of `groups` histograms (groups x M x (2n+1)) and, with
 // groups >= 2, the relative standard error of it: the sample standard
 // deviation of the group estimates over their mean and sqrt(groups) (NaN
@@ -424,17 +443,18 @@ double pt_estimate_from_hist(int variant, int n, int M, const double* beta, cons
 double pt_pooled_estimate(int variant, int n, int M, const double* beta, int groups,
                           const uint64_t* ghist, double* ratios, double* rel_stderr) {
   const size_t per = (size_t)M * (2 * n + 1);
+  const PtWeights weights = pt_weights(variant, n, M, beta);
   std::vector<uint64_t> pooled(per, 0);
   for (int g = 0; g < groups; ++g)
     for (size_t i = 0; i < per; ++i) pooled[i] += ghist[(size_t)g * per + i];
-  const double est = pt_estimate_from_hist(variant, n, M, beta, pooled.data(), ratios);
+  const double est = estimate_with(weights, n, M, pooled.data(), ratios);
   if (rel_stderr) {
     *rel_stderr = 0.0;
     if (groups > 1) {
       std::vector<double> eg(groups);
       double mean = 0.0;
       for (int g = 0; g < groups; ++g) {
-        eg[g] = pt_estimate_from_hist(variant, n, M, beta, ghist + (size_t)g * per, nullptr);
+        eg[g] = estimate_with(weights, n, M, ghist + (size_t)g * per, nullptr);
         mean += eg[g] / groups;
       }
       double var = 0.0;
