@@ -25,119 +25,167 @@ __device__ __forceinline__ void ladder_pair_sync(int lw) {
     asm volatile("bar.sync 2, 64;" ::: "memory");
 }
 
+// Shared-memory accesses by 32-bit address.
+__device__ __forceinline__ int pt_lds8(unsigned a) {
+  int v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void pt_sts8(unsigned a, int v) {
+  asm volatile("st.shared.u8 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void pt_hist_add(unsigned a, unsigned inc) {
+  unsigned v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "r"(v + inc) : "memory");
+}
+
+// A rung's acceptance thresholds: T - 1 in 32 bits (accept iff word <= T - 1;
+// T = 2^32, "always", included), or T itself in 64 bits where some threshold
+// of the run is 0 ("never") or a pair has a single slot (GEN).
+template <bool GEN>
+struct PtThr {
+  typedef unsigned type;
+  __device__ __forceinline__ static bool take(unsigned w, unsigned t) { return w <= t; }
+};
+template <>
+struct PtThr<true> {
+  typedef unsigned long long type;
+  __device__ __forceinline__ static bool take(unsigned w, unsigned long long t) {
+    return (unsigned long long)w < t;
+  }
+};
+
 // Per-warp view of one ladder's tables and this lane's per-rung constants.
 // A ladder has W warps (W = 1: up to 32 rungs; W = 2: up to 64): lane j of
 // warp h serves rung 32 h + j, and the tables have C = 32 W columns.
+template <bool GEN>
 struct PtLane {
-  unsigned short* hist;                 // [E][C]
-  unsigned char* slot;                  // [k][C], k = 1..n
-  unsigned char* occ;                   // [b][C]
-  unsigned char* dir;                   // [C]: the last end of the ladder each column's
+  typedef typename PtThr<GEN>::type Thr;
+  unsigned hist;                        // shared address of [E][rung], this rung's column
+  unsigned slot;                        // [k - 1][C], pair k = 1..n
+  unsigned occ;                         // [b][C]
+  unsigned dir;                         // [C]: the last end of the ladder each column's
                                         // configuration sat at (0 none, 1 rung 0, 2 rung M-1)
-  unsigned long long tm1, tm2;          // move thresholds at this lane's rung, dE = 1, 2
-  const unsigned long long* tswap;      // [M][bins+1]
-  int rung, M, n, delta, bins, nb;
+  Thr tm1, tm2;                         // move thresholds at this lane's rung, dE = 1, 2
+  const Thr* tswap;                     // [M][bins+1]
+  int rung, M, n, delta, bins;
+  // the exchange of iterations of parity 0 and 1: the partner's lane, the
+  // lower rung's lane, the pair's row of tswap, and whether this lane is the
+  // lower one and the pair exists
+  int partner[2], low_lane[2], row[2];
+  bool lower[2], valid[2];
   unsigned burnin;
   bool active;                          // rung < M
   // W = 2: the rung pair (31, 32) across the two warps meets in `xs`
   // (double-buffered by iteration parity) at named barrier `bar`
-  unsigned* xs;                         // [2][3]: pk of rung 31, its word 3, pk of rung 32
+  unsigned* xs;                         // [2][3]: state of rung 31, its word 3, state of rung 32
   int lw;                               // ladder of the block
 };
 
-// Iteration t at rung S.rung, Philox block wc: the energy statistic, one
-// Metropolis move of the configuration in column c (energy E), then the
-// exchange of this rung's pair (j, j+1), j = t mod 2.  Branch-free: every
-// store and the threshold load happen, with unchanged values where a move
-// or exchange is rejected.  With two warps a ladder, the pair (31, 32) is
-// exchanged through shared memory on odd iterations, after a barrier of the
-// two warps (also the point where the columns that change warp become the
-// other warp's).  TRIPS: first the lanes at the two ends of the ladder look
-// at their configurations -- at rung 0 a configuration that has reached rung
-// M-1 since it was last there completes a round trip (counted from `burnin`
-// on), at rung M-1 one that came from rung 0 is marked.
-template <int W, bool TRIPS>
-__device__ __forceinline__ void pt_step(const PtLane& S, const uint4 wc, const unsigned t, int& c,
-                                        int& E, unsigned& accm, unsigned& accs, unsigned& trips) {
+// Iteration t (parity PAR) at rung S.rung, Philox block wc: the energy
+// statistic, one Metropolis move of the configuration here (st = energy << 8 |
+// column), then the exchange of this rung's pair (j, j+1), j = t mod 2.  The
+// stores of a move are predicated, everything else happens with unchanged
+// values where a move or exchange is rejected.  With two warps a ladder, the
+// pair (31, 32) is exchanged through shared memory on odd iterations, after a
+// barrier of the two warps (also the point where the columns that change warp
+// become the other warp's).  TRIPS: first the lanes at the two ends of the
+// ladder look at their configurations -- at rung 0 a configuration that has
+// reached rung M-1 since it was last there completes a round trip (counted
+// from `burnin` on), at rung M-1 one that came from rung 0 is marked.
+template <int W, int PAR, bool TRIPS, bool GEN>
+__device__ __forceinline__ void pt_step(const PtLane<GEN>& S, const uint4 wc, const unsigned t,
+                                        unsigned& st, unsigned& accm, unsigned& accs,
+                                        unsigned& trips) {
   constexpr int C = 32 * W;
+  const unsigned c = st & 0xffu;
   if constexpr (TRIPS) {
     if (S.rung == 0 || S.rung == S.M - 1) {
-      const int dv = S.dir[c];
+      const int dv = pt_lds8(S.dir + c);
       if (S.rung == 0) {
         trips += (unsigned)(dv == 2 && t >= S.burnin);
-        S.dir[c] = 1;
+        pt_sts8(S.dir + c, 1);
       } else if (dv == 1) {
-        S.dir[c] = 2;
+        pt_sts8(S.dir + c, 2);
       }
     }
   }
-  unsigned xw_lo = __shfl_up_sync(0xffffffffu, wc.w, 1);          // word 3 of rung - 1
-  S.hist[E * C + S.rung] += (unsigned short)(S.active && t >= S.burnin);
-  // Metropolis move: pair k to another start slot
-  const int k = 1 + (int)__umulhi(wc.x, (unsigned)S.n);
-  const int d = k + S.delta;
+  pt_hist_add(S.hist + (st >> 8) * (2 * C), (unsigned)(S.active && t >= S.burnin));
+  // Metropolis move: pair k0 + 1 to another start slot
+  const int k0 = (int)__umulhi(wc.x, (unsigned)S.n);
+  const int d = k0 + 1 + S.delta;
   const int L = S.bins - d;
-  unsigned char* sk = &S.slot[k * C + c];
-  const int s_old = *sk;
+  const unsigned ask = S.slot + (unsigned)k0 * C + c;
+  const int s_old = pt_lds8(ask);
+  int s_new = (int)__umulhi(wc.y, (unsigned)(L - 1));
+  s_new += s_new >= s_old;
   // L = 1 (Langford n = 2, k = 2): no other slot; s_new = s_old keeps the
   // reads inside the table and the move is never taken
-  int s_new = s_old;
-  if (L >= 2) {
-    s_new = (int)__umulhi(wc.y, (unsigned)(L - 1));
-    s_new += s_new >= s_old;
+  if constexpr (GEN) {
+    if (L < 2) s_new = s_old;
   }
-  unsigned char* o1 = &S.occ[s_old * C + c];
-  unsigned char* o2 = &S.occ[(s_old + d) * C + c];
-  unsigned char* o3 = &S.occ[s_new * C + c];
-  unsigned char* o4 = &S.occ[(s_new + d) * C + c];
-  const int a1 = *o1, a2 = *o2, a3 = *o3, a4 = *o4;
+  const unsigned ob = S.occ + c, dC = (unsigned)d * C;
+  const unsigned o1 = ob + (unsigned)s_old * C, o2 = o1 + dC;
+  const unsigned o3 = ob + (unsigned)s_new * C, o4 = o3 + dC;
+  const int a1 = pt_lds8(o1), a2 = pt_lds8(o2), a3 = pt_lds8(o3), a4 = pt_lds8(o4);
   // dE: taking the pair out empties the bins it was alone in; putting it
   // back fills the empty bins it lands on (a new bin may be the old pair's
-  // other bin: s_new = s_old + d or s_new + d = s_old)
-  const int b3 = a3 - (s_new == s_old + d);
-  const int b4 = a4 - (s_new + d == s_old);
-  const int dE = (a1 == 1) + (a2 == 1) - (b3 == 0) - (b4 == 0);
-  const unsigned long long thr = dE <= 0 ? (1ull << 32) : (dE == 1 ? S.tm1 : S.tm2);
-  const bool acc = S.active && L >= 2 && (unsigned long long)wc.z < thr;
+  // other bin).  The four counts side by side (each below 128): byte 0x81 - a
+  // has its top bit set iff a <= 1 (a >= 1), 0x80 - b iff b == 0
+  const int b3 = a3 - (o3 == o2);
+  const int b4 = a4 - (o4 == o1);
+  const unsigned four = (unsigned)(a1 + (a2 << 8)) + ((unsigned)(b3 + (b4 << 8)) << 16);
+  const int dE = __dp4a((int)(((0x80808181u - four) >> 7) & 0x01010101u), (int)0xFFFF0101, 0);
+  bool acc;
+  if constexpr (GEN) {
+    const unsigned long long thr = dE <= 0 ? (1ull << 32) : (dE == 1 ? S.tm1 : S.tm2);
+    acc = S.active && L >= 2 && PtThr<GEN>::take(wc.z, thr);
+  } else {
+    const unsigned thr = dE == 1 ? S.tm1 : S.tm2;
+    acc = S.active && (dE <= 0 || PtThr<GEN>::take(wc.z, thr));
+  }
   // counts written in this order are right when bins coincide: o3 == o2
   // ends at b3 + 1 = a2, o4 == o1 at b4 + 1 = a1
-  const int ai = acc;
-  *o1 = (unsigned char)(a1 - ai);
-  *o2 = (unsigned char)(a2 - ai);
-  *o3 = (unsigned char)(acc ? b3 + 1 : a3);
-  *o4 = (unsigned char)(acc ? b4 + 1 : a4);
-  *sk = (unsigned char)(acc ? s_new : s_old);
-  E += acc ? dE : 0;
-  accm += ai;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t"
+      "@p st.shared.u8 [%1], %5;\n\t@p st.shared.u8 [%2], %6;\n\t"
+      "@p st.shared.u8 [%3], %7;\n\t@p st.shared.u8 [%4], %8;\n\t"
+      "@p st.shared.u8 [%9], %10;\n\t}" ::"r"((unsigned)acc),
+      "r"(o1), "r"(o2), "r"(o3), "r"(o4), "r"(a1 - 1), "r"(a2 - 1), "r"(b3 + 1), "r"(b4 + 1),
+      "r"(ask), "r"(s_new)
+      : "memory");
+  if (acc) st += (unsigned)(dE * 256);
+  accm += (unsigned)acc;
   __syncwarp();
   // exchange: both lanes of a pair take the same decision from the lower
   // rung's word 3
-  const int pk = (E << 8) | c;
-  int dn = __shfl_down_sync(0xffffffffu, pk, 1);
-  int up = __shfl_up_sync(0xffffffffu, pk, 1);
-  if constexpr (W == 2) {
-    if (t & 1u) {                                     // the pair (31, 32) is active
-      unsigned* x = S.xs + 3 * (int)((t >> 1) & 1u);
-      if (S.rung == 31) { x[0] = (unsigned)pk; x[1] = wc.w; }
-      if (S.rung == 32) x[2] = (unsigned)pk;
-      ladder_pair_sync(S.lw);
-      if (S.rung == 31) dn = (int)x[2];
-      if (S.rung == 32) { up = (int)x[0]; xw_lo = x[1]; }
-    }
+  unsigned o = __shfl_sync(0xffffffffu, st, S.partner[PAR]);
+  unsigned xw = __shfl_sync(0xffffffffu, wc.w, S.low_lane[PAR]);
+  if constexpr (W == 2 && PAR == 1) {
+    // the pair (31, 32) is active
+    unsigned* x = S.xs + 3 * (int)((t >> 1) & 1u);
+    if (S.rung == 31) { x[0] = st; x[1] = wc.w; }
+    if (S.rung == 32) x[2] = st;
+    ladder_pair_sync(S.lw);
+    if (S.rung == 31) o = x[2];
+    if (S.rung == 32) { o = x[0]; xw = x[1]; }
   }
-  const int par = (S.rung ^ (int)t) & 1;              // 0: lower rung of its pair, 1: upper
-  const int row = S.rung - par;                       // the pair (row, row + 1)
-  const bool valid = row >= 0 && row + 1 < S.M;
-  const int o = par ? up : dn;
-  const int de = par ? (o >> 8) - E : E - (o >> 8);
-  const unsigned xw = par ? xw_lo : wc.w;
-  const unsigned long long T = __ldg(S.tswap + (valid ? row : 0) * S.nb + (de > 0 ? de : 0));
-  const bool dec = valid && (de <= 0 || (unsigned long long)xw < T);
-  c = dec ? (o & 0xff) : c;
-  E = dec ? (o >> 8) : E;
-  accs += dec && !par;
+  const int diff = (int)(st >> 8) - (int)(o >> 8);
+  const int de = S.lower[PAR] ? diff : -diff;
+  const typename PtThr<GEN>::type T = __ldg(S.tswap + S.row[PAR] + (de > 0 ? de : 0));
+  const bool dec = S.valid[PAR] && (de <= 0 || PtThr<GEN>::take(xw, T));
+  st = dec ? o : st;
+  accs += (unsigned)(dec && S.lower[PAR]);
 }
 
+// Bound by issue and the multiply pipe (65 and 70 % busy under ncu, 135 warp
+// instructions an iteration, 40 of them Philox): 32 rungs x 4096 ladders of
+// S(20) in 711 ns an iteration; with two-role exchanges, 64-bit thresholds and
+// unpredicated stores (165 instructions) 853 ns.  64 rungs of L(32): 1601 and
+// 1864 ns; 256 ladders, bound by one iteration's latency, 221 and 272 ns.  One
+// ladder a CTA, for an even spread over the SMs, measured the same.
+//
 // W warps = one ladder (W = 1: up to 32 rungs, W = 2: up to 64); persistent
 // over ladders.  Per iteration t, in the order of Algorithm 2: the energy
 // statistics of every rung (after burn-in), one Metropolis move per
@@ -146,10 +194,10 @@ __device__ __forceinline__ void pt_step(const PtLane& S, const uint4 wc, const u
 // c of the configuration now at that rung and its energy E.  TRIPS: the
 // round trips of the configurations between the ends of the ladder are
 // counted into *trips_g.
-template <int W, bool TRIPS>
+template <int W, bool TRIPS, bool GEN>
 __global__ void __launch_bounds__(128, 7)
-    pt_kernel(PtParams p, const unsigned long long* __restrict__ tmove_g,
-              const unsigned long long* __restrict__ tswap_g, unsigned long long* hist_g,
+    pt_kernel(PtParams p, const typename PtThr<GEN>::type* __restrict__ tmove_g,
+              const typename PtThr<GEN>::type* __restrict__ tswap_g, unsigned long long* hist_g,
               unsigned long long* accm_g, unsigned long long* accs_g, unsigned char* final_slots,
               unsigned long long* trips_g) {
   constexpr int C = 32 * W;
@@ -160,36 +208,45 @@ __global__ void __launch_bounds__(128, 7)
   const int rung = 32 * h + lane;
   const int M = p.M, n = p.n, bins = p.bins, nb = bins + 1;
   unsigned char* wbase = pt_smem + (size_t)lw * pt_ladder_bytes(n, W);
-  PtLane S;
-  S.hist = (unsigned short*)wbase;
-  S.slot = wbase + pt_hist_bytes(n, W);
-  S.occ = S.slot + (n + 1) * C;
-  S.dir = S.occ + bins * C;
+  unsigned short* hist = (unsigned short*)wbase;      // [E][rung]
+  unsigned char* slot = wbase + pt_hist_bytes(n, W);  // [k][column], k = 1..n
+  unsigned char* occ = slot + (n + 1) * C;            // [bin][column]
+  unsigned char* dir = occ + bins * C;                // [column]
+  PtLane<GEN> S;
+  S.hist = (unsigned)__cvta_generic_to_shared(hist + rung);
+  S.slot = (unsigned)__cvta_generic_to_shared(slot + C);
+  S.occ = (unsigned)__cvta_generic_to_shared(occ);
+  S.dir = (unsigned)__cvta_generic_to_shared(dir);
   S.rung = rung;
   S.M = M;
   S.n = n;
   S.delta = p.delta;
   S.bins = bins;
-  S.nb = nb;
   S.burnin = p.burnin;
   S.active = rung < M;
-  S.tm1 = S.active ? __ldg(&tmove_g[rung * 2]) : 0ull;
-  S.tm2 = S.active ? __ldg(&tmove_g[rung * 2 + 1]) : 0ull;
+  S.tm1 = S.active ? __ldg(&tmove_g[rung * 2]) : 0;
+  S.tm2 = S.active ? __ldg(&tmove_g[rung * 2 + 1]) : 0;
   S.tswap = tswap_g;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    S.lower[q] = (rung & 1) == q;
+    S.partner[q] = S.lower[q] ? lane + 1 : lane - 1;
+    S.low_lane[q] = S.lower[q] ? lane : lane - 1;
+    const int row = S.lower[q] ? rung : rung - 1;      // the pair (row, row + 1)
+    S.valid[q] = row >= 0 && row + 1 < M;
+    S.row[q] = (S.valid[q] ? row : 0) * nb;
+  }
   S.xs = xslot[lw & 1];
   S.lw = lw;
-  unsigned short* hist = S.hist;
-  unsigned char* slot = S.slot;
-  unsigned char* occ = S.occ;
   const bool active = S.active;
   const int lpb = p.warps_per_block / W;              // ladders per block
   for (int ladder = blockIdx.x * lpb + lw; ladder < p.ladders; ladder += gridDim.x * lpb) {
     for (int e = 0; e < nb; ++e) hist[e * C + rung] = 0;
     for (int b = 0; b < bins; ++b) occ[b * C + rung] = 0;
     for (int k = 0; k <= n; ++k) slot[k * C + rung] = 0;
-    S.dir[rung] = 0;
+    dir[rung] = 0;
     // column `rung` <- the configuration that starts at that rung
-    int c = rung, E = 0;
+    int E = 0;
     unsigned accm = 0, accs = 0, trips = 0;
     if (active) {
       for (int k = 1; k <= n; ++k) {
@@ -203,6 +260,7 @@ __global__ void __launch_bounds__(128, 7)
       }
       for (int b = 0; b < bins; ++b) E += occ[b * C + rung] == 0;
     }
+    unsigned st = ((unsigned)E << 8) | (unsigned)rung;
     __syncwarp();
     for (unsigned long long t0 = 0; t0 < p.iters; t0 += kPtFlush) {
       const unsigned t1 = (unsigned)(t0 + kPtFlush < p.iters ? t0 + kPtFlush : p.iters);
@@ -212,11 +270,11 @@ __global__ void __launch_bounds__(128, 7)
       unsigned t = (unsigned)t0;
       for (; t + 1 < t1; t += 2) {
         const uint4 wb = philox4x32_10_rk(make_uint4(t + 1u, (unsigned)rung, (unsigned)ladder, 2u), p.rk);
-        pt_step<W, TRIPS>(S, wa, t, c, E, accm, accs, trips);
+        pt_step<W, 0, TRIPS, GEN>(S, wa, t, st, accm, accs, trips);
         wa = philox4x32_10_rk(make_uint4(t + 2u, (unsigned)rung, (unsigned)ladder, 2u), p.rk);
-        pt_step<W, TRIPS>(S, wb, t + 1, c, E, accm, accs, trips);
+        pt_step<W, 1, TRIPS, GEN>(S, wb, t + 1, st, accm, accs, trips);
       }
-      if (t < t1) pt_step<W, TRIPS>(S, wa, t, c, E, accm, accs, trips);
+      if (t < t1) pt_step<W, 0, TRIPS, GEN>(S, wa, t, st, accm, accs, trips);
       if (t1 < p.iters && active) {                // 16-bit counters: flush this rung's column
         unsigned long long* hist_l =
             hist_g + (size_t)pt_group(ladder, p.ladders, p.groups) * M * nb;
@@ -239,7 +297,7 @@ __global__ void __launch_bounds__(128, 7)
       if (TRIPS && trips) atomicAdd(trips_g, (unsigned long long)trips);
       if (final_slots)
         for (int k = 1; k <= n; ++k)
-          final_slots[((size_t)ladder * M + rung) * n + (k - 1)] = slot[k * C + c];
+          final_slots[((size_t)ladder * M + rung) * n + (k - 1)] = slot[k * C + (st & 0xffu)];
     }
     if constexpr (W == 2) ladder_pair_sync(lw);
     __syncwarp();
@@ -301,6 +359,12 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
       for (int de = 1; de <= bins; ++de)
         ts[j * nb + de] = accept_threshold((beta[j + 1] - beta[j]) * (double)de);
   }
+  // a threshold of 0 ("never") or a pair with one slot needs the general form
+  bool gen = bins - (n + (variant == SK_LANGFORD ? 1 : 0)) < 2;
+  for (int j = 0; j < M; ++j) {
+    gen = gen || tm[j * 2] == 0 || tm[j * 2 + 1] == 0;
+    for (int de = 1; j + 1 < M && de <= bins; ++de) gen = gen || ts[j * nb + de] == 0;
+  }
   PtParams p;
   p.n = n;
   p.delta = variant == SK_LANGFORD ? 1 : 0;
@@ -329,8 +393,14 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   unsigned long long* d = (unsigned long long*)cs.dmem();
   unsigned long long* hthr = (unsigned long long*)cs.hmem();
   unsigned long long* hh = hthr + n_thr;
-  std::copy(tm.begin(), tm.end(), hthr);
-  std::copy(ts.begin(), ts.end(), hthr + tm.size());
+  if (gen) {
+    std::copy(tm.begin(), tm.end(), hthr);
+    std::copy(ts.begin(), ts.end(), hthr + tm.size());
+  } else {                                       // T - 1 (entries de = 0 are never compared)
+    unsigned *h1 = (unsigned*)hthr, *h2 = (unsigned*)(hthr + tm.size());
+    for (size_t i = 0; i < tm.size(); ++i) h1[i] = (unsigned)(tm[i] - 1);
+    for (size_t i = 0; i < ts.size(); ++i) h2[i] = (unsigned)(ts[i] - 1);
+  }
   unsigned long long* dtm = d;
   unsigned long long* dts = dtm + tm.size();
   unsigned long long* dh = dts + ts.size();
@@ -342,8 +412,11 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   if (e == cudaSuccess) e = cudaMemsetAsync(dh, 0, n_out * 8, s);
   const size_t smem = pt_smem_bytes(n, W, p.warps_per_block);
   const bool trips = round_trips != nullptr;
-  const auto kernel = W == 2 ? (trips ? pt_kernel<2, true> : pt_kernel<2, false>)
-                             : (trips ? pt_kernel<1, true> : pt_kernel<1, false>);
+  const void* kernel =
+      gen ? (W == 2 ? (trips ? (const void*)pt_kernel<2, true, true> : (const void*)pt_kernel<2, false, true>)
+                    : (trips ? (const void*)pt_kernel<1, true, true> : (const void*)pt_kernel<1, false, true>))
+          : (W == 2 ? (trips ? (const void*)pt_kernel<2, true, false> : (const void*)pt_kernel<2, false, false>)
+                    : (trips ? (const void*)pt_kernel<1, true, false> : (const void*)pt_kernel<1, false, false>));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, per_sm = 0;
@@ -356,10 +429,9 @@ int pt_run_impl(int variant, int n, int M, const double* beta, int L, uint64_t i
   const int need = (L + lpb - 1) / lpb;
   if (grid > need) grid = need;
   if (e == cudaSuccess) e = cudaEventRecord(cs.e0(), s);
-  if (e == cudaSuccess) {
-    kernel<<<grid, 32 * p.warps_per_block, smem, s>>>(p, dtm, dts, dh, dam, das, dfin, dtrips);
-    e = cudaGetLastError();
-  }
+  void* args[] = {&p, &dtm, &dts, &dh, &dam, &das, &dfin, &dtrips};
+  if (e == cudaSuccess)
+    e = cudaLaunchKernel(kernel, dim3(grid), dim3(32 * p.warps_per_block), args, smem, s);
   if (e == cudaSuccess) e = cudaEventRecord(cs.e1(), s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hh, dh, n_out * 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && final_slots)
