@@ -629,7 +629,7 @@ class Mlp:
     def forward(self, slots):
         np = _np()
         s = np.ascontiguousarray(slots, dtype=np.uint8)
-        out = np.zeros((s.shape[0], self.n_moves), dtype=np.float32)
+        out = np.empty((s.shape[0], self.n_moves), dtype=np.float32)
         st = lib().sk_mlp_forward(self.handle, s.ctypes.data, s.shape[0], out.ctypes.data)
         if st != SK_OK:
             raise SkolemError(st, "sk_mlp_forward")
@@ -640,7 +640,7 @@ class Mlp:
         bf16 bit patterns (uint16, B x n_moves)."""
         np = _np()
         s = np.ascontiguousarray(slots, dtype=np.uint8)
-        out = np.zeros((s.shape[0], self.n_moves), dtype=np.uint16)
+        out = np.empty((s.shape[0], self.n_moves), dtype=np.uint16)
         st = lib().sk_mlp_forward_bf16(self.handle, s.ctypes.data, s.shape[0], out.ctypes.data)
         if st != SK_OK:
             raise SkolemError(st, "sk_mlp_forward_bf16")

@@ -116,38 +116,29 @@ namespace sk {
 // One warp per state: target t(m) ~ exp(-beta* dE(m)) over the valid moves,
 // q = masked softmax of the logits, dZ = (q - t) / B, loss += -sum t log q / B.
 // The state's logit row is loaded at once into registers (CH chunks of 256
-// moves, lane l holding moves 256 c + 8 l .. + 7, two 16-byte loads a chunk);
-// the pair and slot of each move come from a per-block table, dE from the
-// state's bin counts in shared memory.  One instantiation per CH = NMp / 256.
+// moves, lane l holding moves 256 c + 8 l .. + 7, two 16-byte loads a chunk),
+// with the moves' pairs and slots (k | slot << 8, map).  dE from bit masks:
+// taking pair k out leaves the bins E_k empty (the empty ones and its own of
+// count 1), so dE = out_k - E_k[s] - E_k[s + d]; a record a pair holds E_k,
+// E_k >> d, out_k and the current slot.  dE takes five values: their target
+// weights are computed once a state (as the five lanes' exponentials and, once
+// the sum is known, quotients) and looked up.  Bound by issue: 2870
+// instructions a state with dE from the bin counts and four exponentials and a
+// division a move 25.4 us for 4096 states of n = 20 (cold), now 17.7 us.  One
+// instantiation per CH = NMp / 256.
 template <int CH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, CH <= 3 ? 4 : 1)
     mlp_loss_kernel(const float* __restrict__ Z, int ldz, const unsigned char* __restrict__ slots,
-                    int B, MoveTable mt, float beta_star, float inv_B, __nv_bfloat16* dZ,
-                    float* loss) {
-  __shared__ unsigned char mk[CH * 256], msl[CH * 256];
-  __shared__ int s_occ[8][2 * kPtMaxN];
-  __shared__ unsigned char s_slot[8][kPtMaxN + 1];
-  for (int m = threadIdx.x; m < CH * 256; m += blockDim.x) {
-    int k = 0, sl = 0;
-    if (m < mt.NM) {                       // the pair with off[k] <= m < off[k+1]
-      int lo = 1, hi = mt.n;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (mt.off[mid] <= m) lo = mid;
-        else hi = mid - 1;
-      }
-      k = lo;
-      sl = m - mt.off[lo];
-    }
-    mk[m] = (unsigned char)k;
-    msl[m] = (unsigned char)sl;
-  }
-  __syncthreads();
+                    const unsigned short* __restrict__ map, int B, int n, int delta, int NM,
+                    float beta_star, float inv_B, __nv_bfloat16* dZ, float* loss) {
+  __shared__ unsigned s_rec[8][kMlpMaxN + 1][8];   // E_k (3 words), E_k >> d (3), out | slot << 8
+  __shared__ int s_occ[8][96];
+  __shared__ float s_te[8][8];                     // target weight of dE = i - 2, then its share
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int b = blockIdx.x * 8 + w;
   if (b >= B) return;
-  const int n = mt.n, NM = mt.NM;
   float z[CH][8];
+  uint4 mv[CH];
   const float* zr = Z + (size_t)b * ldz;
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
@@ -157,38 +148,83 @@ __global__ void __launch_bounds__(256)
       a = __ldg((const float4*)(zr + m0));
       e = __ldg((const float4*)(zr + m0 + 4));
     }
+    mv[c] = __ldg((const uint4*)(map + m0));
     z[c][0] = a.x; z[c][1] = a.y; z[c][2] = a.z; z[c][3] = a.w;
     z[c][4] = e.x; z[c][5] = e.y; z[c][6] = e.z; z[c][7] = e.w;
   }
-  for (int i = lane; i < 2 * n; i += 32) s_occ[w][i] = 0;
-  if (lane == 0) s_slot[w][0] = 0;
+  for (int i = lane; i < 96; i += 32) s_occ[w][i] = 0;
   __syncwarp();
-  for (int k = 1 + lane; k <= n; k += 32) {           // lane k-1 places pair k
-    const int s = slots[(size_t)b * n + (k - 1)];
-    s_slot[w][k] = (unsigned char)s;
-    atomicAdd(&s_occ[w][s], 1);
-    atomicAdd(&s_occ[w][s + k + mt.delta], 1);
+  int sk[2];                                          // lane k-1: pair k's slot (and k + 32's)
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = 1 + lane + 32 * h;
+    sk[h] = 0;
+    if (k <= n) {
+      sk[h] = slots[(size_t)b * n + (k - 1)];
+      if (sk[h] < 2 * n - (k + delta)) {   // a start outside the pair's range counts nothing
+        atomicAdd(&s_occ[w][sk[h]], 1);
+        atomicAdd(&s_occ[w][sk[h] + k + delta], 1);
+      }
+    }
   }
   __syncwarp();
-  // valid moves and their dE
-  int de[CH][8];
-  unsigned vb[CH];
+  unsigned e0[3], e1[3];                              // bins of count 0, of count 1
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {
+    const int o = s_occ[w][lane + 32 * h];
+    e0[h] = __ballot_sync(0xffffffffu, o == 0);
+    e1[h] = __ballot_sync(0xffffffffu, o == 1);
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = 1 + lane + 32 * h;
+    if (k <= n) {
+      const int d = k + delta, p[2] = {sk[h], sk[h] + d};
+      unsigned x[4] = {e0[0], e0[1], e0[2], 0u};
+      unsigned out = 0;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const unsigned own = p[i] >> 5 == j ? e1[j] & (1u << (p[i] & 31)) : 0u;
+          x[j] |= own;
+          out += own != 0u;
+        }
+      unsigned* r = s_rec[w][k];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        r[j] = x[j];
+        // E_k >> d, d <= 41
+        const unsigned lo = d < 32 ? x[j] : x[j + 1];
+        const unsigned hi = d < 32 ? x[j + 1] : (j < 2 ? x[j + 2] : 0u);
+        r[3 + j] = __funnelshift_r(lo, hi, (unsigned)d & 31u);
+      }
+      r[6] = out | ((unsigned)sk[h] << 8);
+    }
+  }
+  if (lane < 8) s_rec[w][0][lane] = 0u;               // padding moves: pair 0 at its slot 0
+  __syncwarp();
+  // per move dE + 2 and whether it is valid, four bits each
+  unsigned dv[CH];
   float zmax = -INFINITY;
   int demin = 1 << 20;
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
-    vb[c] = 0;
+    dv[c] = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int m = c * 256 + lane * 8 + i;
-      const int k = mk[m], sl = msl[m];
-      const int sk = s_slot[w][k];
-      const bool v = m < NM && sl != sk;     // padding: pair 0, slot 0 = s_slot[0]
-      de[c][i] = v ? move_delta_e(s_occ[w], sk, k + mt.delta, sl) : 0;
-      vb[c] |= (unsigned)v << i;
+      const unsigned word = (&mv[c].x)[i >> 1];
+      const unsigned ks = (i & 1) ? word >> 16 : word & 0xffffu;
+      const unsigned k = ks & 0xffu, sl = ks >> 8;
+      const unsigned* r = s_rec[w][k];
+      const unsigned meta = r[6], wi = sl >> 5;
+      const int de = (int)(meta & 3u) - (int)((r[wi] >> (sl & 31u)) & 1u) -
+                     (int)((r[3 + wi] >> (sl & 31u)) & 1u);
+      const bool v = sl != meta >> 8;
+      dv[c] |= ((unsigned)(de + 2) | (v ? 8u : 0u)) << (4 * i);
       if (v) {
         zmax = fmaxf(zmax, z[c][i]);
-        demin = min(demin, de[c][i]);
+        demin = min(demin, de);
       }
     }
   }
@@ -196,18 +232,23 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int o = 16; o; o >>= 1) demin = min(demin, __shfl_xor_sync(0xffffffffu, demin, o));
   const float wmax = -beta_star * (float)demin;
+  if (lane < 5) s_te[w][lane] = __expf(-beta_star * (float)(lane - 2) - wmax);
+  __syncwarp();
   float sq = 0.f, stt = 0.f;
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if ((vb[c] >> i) & 1u) {
+      if ((dv[c] >> (4 * i + 3)) & 1u) {
         sq += __expf(z[c][i] - zmax);
-        stt += __expf(-beta_star * (float)de[c][i] - wmax);
+        stt += s_te[w][(dv[c] >> (4 * i)) & 7u];
       }
   sq = warp_sum(sq);
   stt = warp_sum(stt);
   const float lse = zmax + __logf(sq);
+  __syncwarp();
+  if (lane < 5) s_te[w][lane] = s_te[w][lane] / stt;
+  __syncwarp();
   float l = 0.f;
   __nv_bfloat16* dz = dZ + (size_t)b * ldz;
 #pragma unroll
@@ -219,9 +260,9 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         g[h] = 0.f;
-        if ((vb[c] >> (i + h)) & 1u) {
+        if ((dv[c] >> (4 * (i + h) + 3)) & 1u) {
           const float q = __expf(z[c][i + h] - lse);
-          const float t = __expf(-beta_star * (float)de[c][i + h] - wmax) / stt;
+          const float t = s_te[w][(dv[c] >> (4 * (i + h))) & 7u];
           g[h] = (q - t) * inv_B;
           l -= t * (z[c][i + h] - lse);
         }
@@ -237,13 +278,12 @@ __global__ void __launch_bounds__(256)
 
 // The loss kernel for the model's move-table size (NMp / 256 chunks).
 static cudaError_t launch_loss(const Mlp& m, int B, float beta_star, float* loss, cudaStream_t s) {
-  const MoveTable mt = move_table(m);
   const dim3 grid((B + 7) / 8), block(256);
   switch (m.NMp / 256) {
 #define SK_LOSS_CASE(c)                                                                     \
   case c:                                                                                   \
-    mlp_loss_kernel<c><<<grid, block, 0, s>>>(m.Z, m.NMp, m.slots, B, mt, beta_star,       \
-                                              1.0f / (float)B, m.dZ, loss);                 \
+    mlp_loss_kernel<c><<<grid, block, 0, s>>>(m.Z, m.NMp, m.slots, m.map, B, m.n, m.delta,  \
+                                              m.NM, beta_star, 1.0f / (float)B, m.dZ, loss); \
     break;
     SK_LOSS_CASE(1) SK_LOSS_CASE(2) SK_LOSS_CASE(3) SK_LOSS_CASE(4) SK_LOSS_CASE(5)
     SK_LOSS_CASE(6) SK_LOSS_CASE(7) SK_LOSS_CASE(8) SK_LOSS_CASE(9) SK_LOSS_CASE(10)
@@ -483,7 +523,9 @@ cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, boo
     e = gemm_tc(t, m.tmA[1], m.tmB[1], m.tmC[1], kTcEpiReluBf16, s);
     if (e != cudaSuccess) return e;
     t.N = m.NMp; t.bias = m.b3;
-    if (logits_bf16) t.nvalid = (m.NM + 7) / 8 * 8;   // the columns tmZb stores
+    // only the move table's columns (of the fp32 logits' last 32-column slab
+    // the rest is stored unwritten; nothing reads it)
+    t.nvalid = (m.NM + 7) / 8 * 8;
     return logits_bf16 ? gemm_tc(t, m.tmA[2], m.tmB[2], m.tmZb, kTcEpiBf16, s)
                        : gemm_tc(t, m.tmA[2], m.tmB[2], m.tmC[2], kTcEpiF32, s);
   }
@@ -760,6 +802,7 @@ int mlp_create(int variant, int n, int max_batch, uint64_t seed, Mlp** out) {
   const size_t o_cp = off; off = al256(off + (B / 128) * (size_t)m->NMp * 4);
   const size_t o_wt = off; off = al256(off + (w1 + w2 + w3) * 2);
   const size_t o_err = off; off = al256(off + 4);
+  const size_t o_map = off; off = al256(off + (size_t)m->NMp * 2);
   char* p = nullptr;
   if (cudaMalloc(&p, off) != cudaSuccess) {
     delete m;
@@ -789,6 +832,7 @@ int mlp_create(int variant, int n, int max_batch, uint64_t seed, Mlp** out) {
   __nv_bfloat16* wt = (__nv_bfloat16*)(p + o_wt);
   m->W1t = wt; m->W2t = wt + w1; m->W3t = wt + w1 + w2;
   m->tc_err = (unsigned*)(p + o_err);
+  m->map = (unsigned short*)(p + o_map);
   m->use_tc = 1;
   m->wt_dirty = 1;
   if (!make_tc_maps(*m)) {          // the driver could not describe the buffers
@@ -812,6 +856,11 @@ int mlp_create(int variant, int n, int max_batch, uint64_t seed, Mlp** out) {
   if (e == cudaSuccess) e = cudaMemset(m->am, 0, m->nparams * 4);
   if (e == cudaSuccess) e = cudaMemset(m->av, 0, m->nparams * 4);
   if (e == cudaSuccess) e = cudaMemset(m->tc_err, 0, 4);
+  std::vector<unsigned short> map(m->NMp, 0);         // padding: pair 0, slot 0
+  for (int k = 1; k <= n; ++k)
+    for (int i = m->off[k]; i < m->off[k + 1]; ++i)
+      map[i] = (unsigned short)(k | (i - m->off[k]) << 8);
+  if (e == cudaSuccess) e = cudaMemcpy(m->map, map.data(), map.size() * 2, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
     f32_to_bf16_kernel<<<256, 256>>>(par, wb, w1 + w2 + w3);
     e = cudaDeviceSynchronize();

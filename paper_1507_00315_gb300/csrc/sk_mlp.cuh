@@ -39,6 +39,7 @@ struct Mlp {
   int use_tc;                                // 1: forward on tcgen05 (default)
   int wt_dirty;                              // transposed copies need a refresh
   unsigned* tc_err;                          // error word of the tcgen05 GEMM
+  unsigned short* map;                       // [NMp] pair | slot << 8 of every move (padding: 0)
   // TMA descriptors of the tcgen05 forward (128-byte swizzle): operands A =
   // X, H1, H2 ([max_batch][K], boxes [128][64]) and B = W1t, W2t, W3t ([N][K],
   // boxes [256][64]); results C = H1, H2 (bf16, boxes [32][64]) and Z (fp32,
