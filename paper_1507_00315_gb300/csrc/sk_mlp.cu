@@ -32,20 +32,24 @@ cudaError_t gemm(const GemmArgs& g, int splits, cudaStream_t s) {
 }
 
 // X[b][i] = occupancy of bin i of state b (0 beyond 2n; n <= 40, so the
-// bins fit a 128-entry histogram).  One warp per
+// bins fit a 128-entry histogram).  With idx, state b is row idx[b] of `all`
+// and its slots are copied to `slots` as well (a minibatch).  One warp per
 // state: the pairs are counted into a shared histogram, then each lane
 // writes four adjacent bf16 inputs (one 8-byte store; a row is 256 bytes).
-__global__ void __launch_bounds__(256) mlp_inputs_kernel(const unsigned char* __restrict__ slots,
-                                                         int B, int n, int delta, int K1,
-                                                         __nv_bfloat16* X) {
+__global__ void __launch_bounds__(256) mlp_inputs_kernel(unsigned char* slots, int B, int n,
+                                                         int delta, int K1, __nv_bfloat16* X,
+                                                         const unsigned char* __restrict__ all,
+                                                         const unsigned* __restrict__ idx) {
   __shared__ unsigned occ[8][128];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * 8 + w;
   if (b >= B) return;
   for (int i = lane; i < 128; i += 32) occ[w][i] = 0;
   __syncwarp();
+  const unsigned char* from = idx ? all + (size_t)idx[b] * n : slots + (size_t)b * n;
   for (int k = 1 + lane; k <= n; k += 32) {
-    const int s = slots[(size_t)b * n + (k - 1)];
+    const int s = from[k - 1];
+    if (idx) slots[(size_t)b * n + (k - 1)] = (unsigned char)s;
     if (s < 2 * n - (k + delta)) {      // a start outside the pair's range counts nothing
       atomicAdd(&occ[w][s], 1u);
       atomicAdd(&occ[w][s + k + delta], 1u);
@@ -508,7 +512,8 @@ cudaError_t gemm_tc(const TcGemmArgs& g, const CUtensorMap& amap, const CUtensor
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, bool inputs_ready,
                             cudaEvent_t before_l2, bool dependent) {
   if (!inputs_ready)
-    mlp_inputs_kernel<<<(B + 7) / 8, 256, 0, s>>>(m.slots, B, m.n, m.delta, m.K1, m.X);
+    mlp_inputs_kernel<<<(B + 7) / 8, 256, 0, s>>>(m.slots, B, m.n, m.delta, m.K1, m.X, nullptr,
+                                                  nullptr);
   if (m.use_tc) {
     cudaError_t e = cudaSuccess;
     if (m.wt_dirty) e = refresh_transposed(m, s);
@@ -583,32 +588,39 @@ __global__ void grad_finish_kernel(const float* __restrict__ ws, int KS, size_t 
   }
 }
 
-// The workspace of the tcgen05 backward for batches up to B: K-major copies
-// TA [256][B] and TB [NMp][B] of the weight-gradient operands, 16 K-split
-// partials of the largest weight gradient, and the bias gradients' column
-// sums of 64-row tiles [B / 64][NMp].  Grown on demand.
+// The workspaces of the tcgen05 backward for batches up to B, one for each of
+// the three weight gradients (they run side by side): K-major copies TA
+// [256][B] and TB [width][B] of the operands, 16 K-split partials, and the bias
+// gradient's column sums of 64-row tiles [B / 64][width]; width = NMp, 256,
+// 256.  Grown on demand.
 struct BwdSpace {
   __nv_bfloat16 *TA, *TB;
   float *WS, *part;
 };
-static cudaError_t bwd_workspace(Mlp& m, int B, BwdSpace* w) {
+static cudaError_t bwd_workspace(Mlp& m, int B, BwdSpace (&w)[3]) {
   auto a256 = [](size_t x) { return (x + 255) / 256 * 256; };
-  const size_t wide = m.NMp > kHidden ? m.NMp : kHidden;
-  const size_t ta = a256((size_t)kHidden * B * 2), tb = a256((size_t)m.NMp * B * 2),
-               ws = a256((size_t)16 * kHidden * wide * 4), pt = (size_t)(B / 64) * wide * 4;
-  if (ta + tb + ws + pt > m.bwd_bytes) {
+  size_t off = 0, at[3][4];
+  for (int i = 0; i < 3; ++i) {
+    const size_t width = i ? kHidden : m.NMp;
+    const size_t bytes[4] = {(size_t)kHidden * B * 2, width * B * 2, (size_t)16 * kHidden * width * 4,
+                             (size_t)(B / 64) * width * 4};
+    for (int j = 0; j < 4; ++j) {
+      at[i][j] = off;
+      off = a256(off + bytes[j]);
+    }
+  }
+  if (off > m.bwd_bytes) {
     if (m.bwd_ws) cudaFree(m.bwd_ws);
     m.bwd_ws = nullptr;
     m.bwd_bytes = 0;
-    cudaError_t e = cudaMalloc(&m.bwd_ws, ta + tb + ws + pt);
+    cudaError_t e = cudaMalloc(&m.bwd_ws, off);
     if (e != cudaSuccess) return e;
-    m.bwd_bytes = ta + tb + ws + pt;
+    m.bwd_bytes = off;
   }
   char* p = (char*)m.bwd_ws;
-  w->TA = (__nv_bfloat16*)p;
-  w->TB = (__nv_bfloat16*)(p + ta);
-  w->WS = (float*)(p + ta + tb);
-  w->part = (float*)(p + ta + tb + ws);
+  for (int i = 0; i < 3; ++i)
+    w[i] = {(__nv_bfloat16*)(p + at[i][0]), (__nv_bfloat16*)(p + at[i][1]), (float*)(p + at[i][2]),
+            (float*)(p + at[i][3])};
   return cudaSuccess;
 }
 
@@ -653,10 +665,12 @@ int splits_for(int K) {
   return sp;
 }
 
-// The side stream of the tcgen05 backward and its four events, made on first use.
-static cudaError_t side_stream(Mlp& m) {
-  if (m.side) return cudaSuccess;
-  cudaError_t e = cudaStreamCreateWithFlags(&m.side, cudaStreamNonBlocking);
+// The side streams of the tcgen05 backward and their events, made on first use.
+static cudaError_t side_streams(Mlp& m) {
+  if (m.side[1]) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i)
+    if (!m.side[i]) e = cudaStreamCreateWithFlags(&m.side[i], cudaStreamNonBlocking);
   for (int i = 0; i < 4 && e == cudaSuccess; ++i)
     e = cudaEventCreateWithFlags(&m.ev[i], cudaEventDisableTiming);
   return e;
@@ -675,38 +689,40 @@ cudaError_t mlp_backward_dev(Mlp& m, int B, float beta_star, cudaStream_t s,
   if (e != cudaSuccess) return e;
   if (m.use_tc) {
     // tcgen05: dH = (dZ W^T) * [H > 0] with W streamed as B, on s; the
-    // weight and bias gradients (K-major copies, a fixed-order K split) on a
-    // side stream, each as soon as its activation gradient exists; s waits
-    // for the side stream at the end
-    BwdSpace w;
-    e = bwd_workspace(m, B, &w);
-    if (e == cudaSuccess) e = side_stream(m);
+    // weight and bias gradients (K-major copies, a fixed-order K split) of the
+    // third and second layers each on a side stream of its own as soon as the
+    // activation gradient exists, the first layer's on s after them; s waits
+    // for the side streams at the end.  (All three on one side stream were the
+    // longest chain of a step: 58 us after the loss, side by side 43.)
+    BwdSpace w[3];
+    e = bwd_workspace(m, B, w);
+    if (e == cudaSuccess) e = side_streams(m);
     if (e != cudaSuccess) return e;
     int dev = 0;
     cudaGetDevice(&dev);
     const int sms = device_sm_count(dev);
     e = cudaEventRecord(m.ev[0], s);                               // dZ
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(m.side, m.ev[0], 0);
-    if (e == cudaSuccess)
-      e = weight_grad_tc(m, B, m.H2, kHidden, m.dZ, m.NMp, m.gW3, m.gb3, w, sms, m.side);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(m.side[0], m.ev[0], 0);
     TcGemmArgs t;
     std::memset(&t, 0, sizeof(t));
     t.M = B; t.N = kHidden; t.K = m.NMp; t.err = m.tc_err; t.aux = m.H2; t.ldaux = kHidden;
-    e = gemm_tc_launch<kTcEpiMaskBf16, true>(t, m.tmBA[0], m.tmBB[0], m.tmBC[0], s);
+    if (e == cudaSuccess)
+      e = gemm_tc_launch<kTcEpiMaskBf16, true>(t, m.tmBA[0], m.tmBB[0], m.tmBC[0], s);
+    if (e == cudaSuccess)
+      e = weight_grad_tc(m, B, m.H2, kHidden, m.dZ, m.NMp, m.gW3, m.gb3, w[0], sms, m.side[0]);
     if (e == cudaSuccess) e = cudaEventRecord(m.ev[1], s);        // dH2
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(m.side, m.ev[1], 0);
-    if (e == cudaSuccess)
-      e = weight_grad_tc(m, B, m.H1, kHidden, m.dH2, kHidden, m.gW2, m.gb2, w, sms, m.side);
-    if (e != cudaSuccess) return e;
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(m.side[1], m.ev[1], 0);
     t.K = kHidden; t.aux = m.H1;
-    e = gemm_tc_launch<kTcEpiMaskBf16, true>(t, m.tmBA[1], m.tmBB[1], m.tmBC[1], s);
-    if (e == cudaSuccess) e = cudaEventRecord(m.ev[2], s);        // dH1
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(m.side, m.ev[2], 0);
     if (e == cudaSuccess)
-      e = weight_grad_tc(m, B, m.X, m.K1, m.dH1, kHidden, m.gW1, m.gb1, w, sms, m.side);
-    if (e == cudaSuccess) e = cudaEventRecord(m.ev[3], m.side);   // every gradient
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, m.ev[3], 0);
+      e = gemm_tc_launch<kTcEpiMaskBf16, true>(t, m.tmBA[1], m.tmBB[1], m.tmBC[1], s);
+    if (e == cudaSuccess)
+      e = weight_grad_tc(m, B, m.H1, kHidden, m.dH2, kHidden, m.gW2, m.gb2, w[1], sms, m.side[1]);
+    if (e == cudaSuccess)
+      e = weight_grad_tc(m, B, m.X, m.K1, m.dH1, kHidden, m.gW1, m.gb1, w[2], sms, s);
+    for (int i = 0; i < 2; ++i) {
+      if (e == cudaSuccess) e = cudaEventRecord(m.ev[2 + i], m.side[i]);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(s, m.ev[2 + i], 0);
+    }
     return e;
   }
   GemmArgs g;
@@ -751,14 +767,6 @@ cudaError_t mlp_backward_dev(Mlp& m, int B, float beta_star, cudaStream_t s,
 }  // namespace sk
 
 namespace sk {
-
-__global__ void gather_slots_kernel(const unsigned char* __restrict__ all, const unsigned* __restrict__ idx,
-                                    int B, int n, unsigned char* out) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= (size_t)B * n) return;
-  const size_t b = i / n, k = i % n;
-  out[i] = all[(size_t)idx[b] * n + k];
-}
 
 static size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -935,12 +943,13 @@ extern "C" int sk_mlp_create(int variant, int n, int max_batch, uint64_t seed, v
 extern "C" void sk_mlp_destroy(void* model) {
   Mlp* m = (Mlp*)model;
   if (!m) return;
-  if (m->side) {
-    cudaStreamSynchronize(m->side);
-    for (int i = 0; i < 4; ++i)
-      if (m->ev[i]) cudaEventDestroy(m->ev[i]);
-    cudaStreamDestroy(m->side);
-  }
+  for (int i = 0; i < 2; ++i)
+    if (m->side[i]) {
+      cudaStreamSynchronize(m->side[i]);
+      cudaStreamDestroy(m->side[i]);
+    }
+  for (int i = 0; i < 4; ++i)
+    if (m->ev[i]) cudaEventDestroy(m->ev[i]);
   if (m->bwd_ws) cudaFree(m->bwd_ws);
   cudaFree(m->block);
   delete m;
@@ -1021,7 +1030,7 @@ extern "C" int sk_mlp_forward(void* model, const uint8_t* slots, int B, float* l
   if (!m || !slots || !logits || B < 1 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   const int Bp = sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, false, false, nullptr, true);
   if (e == cudaSuccess)
     e = cudaMemcpy2D(logits, (size_t)m->NM * 4, m->Z, (size_t)m->NMp * 4, (size_t)m->NM * 4, B,
                      cudaMemcpyDeviceToHost);
@@ -1037,7 +1046,7 @@ extern "C" int sk_mlp_forward_bf16(void* model, const uint8_t* slots, int B, uin
   if (!m || !slots || !logits || B < 1 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   const int Bp = sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, true);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, true, false, nullptr, true);
   if (e == cudaSuccess)
     e = cudaMemcpy2D(logits, (size_t)m->NM * 2, m->Z, (size_t)m->NMp * 2, (size_t)m->NM * 2, B,
                      cudaMemcpyDeviceToHost);
@@ -1054,7 +1063,7 @@ extern "C" int sk_mlp_loss_grad(void* model, const uint8_t* slots, int B, float 
   if (!m || !slots || B < 128 || B % 128 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, B, nullptr);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, B, nullptr, false, false, nullptr, true);
   if (e == cudaSuccess) e = sk::mlp_backward_dev(*m, B, beta_star, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return sk::cuda_status(e);
@@ -1102,10 +1111,9 @@ int mlp_train_impl(Mlp& m, const uint8_t* states, uint64_t count, int epochs, in
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // perm is reused next epoch
     if (e == cudaSuccess) e = cudaMemsetAsync(dloss, 0, steps * sizeof(float), s);
     for (uint64_t st = 0; st < steps && e == cudaSuccess; ++st) {
-      const size_t tot = (size_t)batch * m.n;
-      gather_slots_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(dstates, didx + st * batch,
-                                                                       batch, m.n, m.slots);
-      e = mlp_forward_dev(m, batch, s);
+      mlp_inputs_kernel<<<(batch + 7) / 8, 256, 0, s>>>(m.slots, batch, m.n, m.delta, m.K1, m.X,
+                                                        dstates, didx + st * batch);
+      e = mlp_forward_dev(m, batch, s, false, true, nullptr, true);
       if (e == cudaSuccess) e = mlp_backward_dev(m, batch, beta_star, s, dloss + st);
       if (e != cudaSuccess) break;
       m.adam_t += 1;

@@ -51,8 +51,8 @@ struct Mlp {
   CUtensorMap tmBA[2], tmBB[2], tmBC[2];
   void* bwd_ws;                              // K-major operand copies + K-split partials
   size_t bwd_bytes;
-  cudaStream_t side;                         // the backward's weight-gradient stream
-  cudaEvent_t ev[4];                         // its fork and join points
+  cudaStream_t side[2];                      // the backward's weight-gradient streams
+  cudaEvent_t ev[4];                         // their fork and join points
   float* Z;
   float* loss;                               // [1]
   float* colpart;                            // [max_batch / 128][NMp]: bias-gradient partials
@@ -92,8 +92,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 // inputs_ready the caller has already written the input rows X.  before_l2:
 // an event the stream waits for between the first and the second layer.
 // dependent: the second and third layers are launched as programmatic
-// dependents of the layer before (they may set up while it finishes; only
-// while the weights stay unchanged, as in a tempering run).
+// dependents of the layer before (they may set up while it finishes).
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16 = false,
                             bool inputs_ready = false, cudaEvent_t before_l2 = nullptr,
                             bool dependent = false);
