@@ -510,7 +510,7 @@ cudaError_t gemm_tc(const TcGemmArgs& g, const CUtensorMap& amap, const CUtensor
 // Forward pass for B (multiple of 128) states whose slots are already in
 // m.slots: X, H1, H2 (bf16) and Z (fp32 logits, or bf16 with logits_bf16).
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, bool inputs_ready,
-                            cudaEvent_t before_l2, bool dependent) {
+                            bool dependent, bool first_dependent) {
   if (!inputs_ready)
     mlp_inputs_kernel<<<(B + 7) / 8, 256, 0, s>>>(m.slots, B, m.n, m.delta, m.K1, m.X, nullptr,
                                                   nullptr);
@@ -521,8 +521,8 @@ cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, boo
     TcGemmArgs t;
     std::memset(&t, 0, sizeof(t));
     t.M = B; t.N = kHidden; t.K = m.K1f; t.bias = m.b1; t.err = m.tc_err;
+    t.pdl = first_dependent ? 1 : 0;
     e = gemm_tc(t, m.tmA[0], m.tmB[0], m.tmC[0], kTcEpiReluBf16, s);
-    if (e == cudaSuccess && before_l2) e = cudaStreamWaitEvent(s, before_l2, 0);
     if (e != cudaSuccess) return e;
     t.K = kHidden; t.bias = m.b2; t.pdl = dependent ? 1 : 0;
     e = gemm_tc(t, m.tmA[1], m.tmB[1], m.tmC[1], kTcEpiReluBf16, s);
@@ -539,7 +539,6 @@ cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, boo
   g.M = B; g.N = kHidden; g.K = m.K1f; g.A = m.X; g.lda = m.K1; g.B = m.W1; g.ldb = kHidden;
   g.C = m.H1; g.ldc = kHidden; g.bias = m.b1;
   cudaError_t e = gemm<false, false, EPI_BF16_RELU>(g, 1, s);
-  if (e == cudaSuccess && before_l2) e = cudaStreamWaitEvent(s, before_l2, 0);
   if (e != cudaSuccess) return e;
   g.K = kHidden; g.A = m.H1; g.lda = kHidden; g.B = m.W2; g.C = m.H2; g.bias = m.b2;
   e = gemm<false, false, EPI_BF16_RELU>(g, 1, s);
@@ -1030,7 +1029,7 @@ extern "C" int sk_mlp_forward(void* model, const uint8_t* slots, int B, float* l
   if (!m || !slots || !logits || B < 1 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   const int Bp = sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, false, false, nullptr, true);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, false, false, true);
   if (e == cudaSuccess)
     e = cudaMemcpy2D(logits, (size_t)m->NM * 4, m->Z, (size_t)m->NMp * 4, (size_t)m->NM * 4, B,
                      cudaMemcpyDeviceToHost);
@@ -1046,7 +1045,7 @@ extern "C" int sk_mlp_forward_bf16(void* model, const uint8_t* slots, int B, uin
   if (!m || !slots || !logits || B < 1 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   const int Bp = sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, true, false, nullptr, true);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, Bp, nullptr, true, false, true);
   if (e == cudaSuccess)
     e = cudaMemcpy2D(logits, (size_t)m->NM * 2, m->Z, (size_t)m->NMp * 2, (size_t)m->NM * 2, B,
                      cudaMemcpyDeviceToHost);
@@ -1063,7 +1062,7 @@ extern "C" int sk_mlp_loss_grad(void* model, const uint8_t* slots, int B, float 
   if (!m || !slots || B < 128 || B % 128 || B > m->max_batch) return SK_EINVAL;
   cudaError_t e;
   sk::upload_states(*m, slots, B, nullptr, &e);
-  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, B, nullptr, false, false, nullptr, true);
+  if (e == cudaSuccess) e = sk::mlp_forward_dev(*m, B, nullptr, false, false, true);
   if (e == cudaSuccess) e = sk::mlp_backward_dev(*m, B, beta_star, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return sk::cuda_status(e);
@@ -1113,7 +1112,7 @@ int mlp_train_impl(Mlp& m, const uint8_t* states, uint64_t count, int epochs, in
     for (uint64_t st = 0; st < steps && e == cudaSuccess; ++st) {
       mlp_inputs_kernel<<<(batch + 7) / 8, 256, 0, s>>>(m.slots, batch, m.n, m.delta, m.K1, m.X,
                                                         dstates, didx + st * batch);
-      e = mlp_forward_dev(m, batch, s, false, true, nullptr, true);
+      e = mlp_forward_dev(m, batch, s, false, true, true);
       if (e == cudaSuccess) e = mlp_backward_dev(m, batch, beta_star, s, dloss + st);
       if (e != cudaSuccess) break;
       m.adam_t += 1;

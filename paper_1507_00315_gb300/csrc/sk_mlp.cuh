@@ -89,13 +89,14 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Forward pass for B (multiple of 128) states whose start slots are in
 // m.slots: X, H1, H2 (bf16) and the logits Z (fp32, [B][NMp]; with
 // logits_bf16, bf16 [B][NMp] in the first half of Z's memory).  With
-// inputs_ready the caller has already written the input rows X.  before_l2:
-// an event the stream waits for between the first and the second layer.
-// dependent: the second and third layers are launched as programmatic
-// dependents of the layer before (they may set up while it finishes).
+// inputs_ready the caller has already written the input rows X.  dependent:
+// the second and third layers are launched as programmatic dependents of the
+// layer before (they may set up while it finishes); first_dependent: the first
+// layer too, of the stream's previous kernel, which must not have written the
+// weights.
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16 = false,
-                            bool inputs_ready = false, cudaEvent_t before_l2 = nullptr,
-                            bool dependent = false);
+                            bool inputs_ready = false, bool dependent = false,
+                            bool first_dependent = false);
 
 // Launch of kernel k as a programmatic dependent of the previous kernel of
 // stream s (it must execute griddepcontrol.wait before it reads what that

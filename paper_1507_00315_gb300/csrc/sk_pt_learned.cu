@@ -24,6 +24,7 @@ namespace sk {
 
 struct LearnedDev {
   int n, delta, M, L, B, nb, NMp;
+  unsigned inv_M;            // ceil(2^32 / M): c / M = the high word of c inv_M (c < 2^32 / M)
   unsigned key0, key1;
   unsigned rk[20];           // Philox round keys of (key0, key1), computed on the host
   unsigned char* slots;      // [B][n] current configurations, c = ladder * M + l
@@ -77,37 +78,37 @@ __device__ __forceinline__ void copy_move_maps(const MoveMaps* g, MoveMaps& mm) 
 
 // A configuration in registers: lane k-1 holds the start slot of pair k,
 // lane k-33 that of pair k > 32 (-1: no such pair).
+// (TWO: n > 32; else sb is not used.)
+template <bool TWO>
 __device__ __forceinline__ void load_slots(const unsigned char* sl, int n, int lane, int& sa,
                                            int& sb) {
   sa = lane < n ? (int)sl[lane] : -1;
-  sb = lane + 32 < n ? (int)sl[lane + 32] : -1;
+  sb = TWO && lane + 32 < n ? (int)sl[lane + 32] : -1;
 }
 
-// The start slot of pair k (1..n) from the lanes that hold the configuration.
+// The start slot of pair k (1..n; the lanes may ask for different pairs) from
+// the lanes that hold the configuration.
+template <bool TWO>
 __device__ __forceinline__ int slot_of(int sa, int sb, int k) {
   const int a = __shfl_sync(0xffffffffu, sa, (k - 1) & 31);
+  if constexpr (!TWO) return a;
   const int b = __shfl_sync(0xffffffffu, sb, (k - 33) & 31);
   return k <= 32 ? a : b;
 }
 
-// The start slot of pair k (1..n, a different pair on each lane) from the
-// lanes that hold the configuration.
-__device__ __forceinline__ int slot_of_lanes(int sa, int sb, int k) {
-  const int a = __shfl_sync(0xffffffffu, sa, (k - 1) & 31);
-  const int b = __shfl_sync(0xffffffffu, sb, (k - 33) & 31);
-  return k <= 32 ? a : b;
-}
-
-// Bin occupancies of the configuration into the warp's counts occ[2n].
-__device__ __forceinline__ void place_occupancy(int sa, int sb, int n, int delta, int* occ,
-                                                int lane) {
-  for (int i = lane; i < 2 * n; i += 32) occ[i] = 0;
+// Bin occupancies of the configuration into the warp's counts occ[128].
+template <bool TWO>
+__device__ __forceinline__ void place_occupancy(int sa, int sb, int delta, int* occ, int lane) {
+  // all the bins the template's orders can have (the array holds 128)
+  occ[lane] = 0;
+  occ[lane + 32] = 0;
+  if constexpr (TWO) occ[lane + 64] = 0;
   __syncwarp();
   if (sa >= 0) {
     atomicAdd(&occ[sa], 1);
     atomicAdd(&occ[sa + lane + 1 + delta], 1);
   }
-  if (sb >= 0) {
+  if (TWO && sb >= 0) {
     atomicAdd(&occ[sb], 1);
     atomicAdd(&occ[sb + lane + 33 + delta], 1);
   }
@@ -120,6 +121,9 @@ __device__ __forceinline__ void place_occupancy(int sa, int sb, int n, int delta
 // chunks of the move table, ceil(NM / 256): the kernels are compiled for
 // each CH up to kLtChunks, so no lane walks chunks the problem does not have.
 constexpr int kLtChunks = kMaxMoves / 256;
+// up to 6 chunks the table is that of an n <= 32 (n = 33 has 1584 moves and more)
+template <int CH>
+constexpr bool kLtTwo = CH > 6;
 template <int CH>
 struct LogitRow {
   uint4 w[CH];
@@ -159,13 +163,16 @@ __device__ __forceinline__ void load_row(const __nv_bfloat16* z, int NM, int lan
 template <int CH>
 __device__ __forceinline__ void row_valid(const MoveMaps& mm, int sa, int sb, int NM, int lane,
                                           unsigned* bits, LogitRow<CH>& r) {
-  for (int i = lane; i < CH * 8; i += 32) bits[i] = 0;
+  if (CH * 8 >= 32 || lane < CH * 8) bits[lane] = 0;
+  if (CH > 4) {
+    for (int i = 32 + lane; i < CH * 8; i += 32) bits[i] = 0;
+  }
   __syncwarp();
   if (sa >= 0) {
     const int m = mm.off[lane + 1] + sa;
     atomicOr(&bits[m >> 5], 1u << (m & 31));
   }
-  if (sb >= 0) {
+  if (kLtTwo<CH> && sb >= 0) {
     const int m = mm.off[lane + 33] + sb;
     atomicOr(&bits[m >> 5], 1u << (m & 31));
   }
@@ -309,11 +316,13 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 // Asynchronous 16-byte copy global -> shared (cp.async, L2 only) and the
 // waits on this thread's own copies.
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                   (unsigned)__cvta_generic_to_shared(dst)),
-               "l"(src)
-               : "memory");
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool on) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t"
+      "@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(
+          (unsigned)__cvta_generic_to_shared(dst)),
+      "l"(src), "r"((unsigned)on)
+      : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
@@ -355,19 +364,19 @@ __device__ __forceinline__ void load_step_in(const LearnedDev& d, const __nv_bfl
                                              const unsigned char* prop_slots, int NM, int c,
                                              int lane, bool first, StepBuf<CH>& buf,
                                              StepIn<CH>& in) {
-  load_slots(prop_slots + (size_t)c * d.n, d.n, lane, in.sa, in.sb);
+  load_slots<kLtTwo<CH>>(prop_slots + (size_t)c * d.n, d.n, lane, in.sa, in.sb);
   in.rung = d.rung[c];
   in.E = d.E[c];
   const __nv_bfloat16* z = Zp + (size_t)c * d.NMp;
 #pragma unroll
   for (int k = 0; k < CH; ++k)
-    if (k * 256 + lane * 8 < NM) cp_async16(&buf.row[k * 32 + lane], z + k * 256 + lane * 8);
+    cp_async16(&buf.row[k * 32 + lane], z + k * 256 + lane * 8, k * 256 + lane * 8 < NM);
   if (!first) {
     const __nv_bfloat16* zc = d.Zcur + (size_t)c * d.NMp;
     const float* pp = d.parts + (size_t)c * CH * 32 + lane;
 #pragma unroll
     for (int k = 0; k < CH; ++k) {
-      if (k * 256 + lane * 8 < NM) cp_async16(&buf.crow[k * 32 + lane], zc + k * 256 + lane * 8);
+      cp_async16(&buf.crow[k * 32 + lane], zc + k * 256 + lane * 8, k * 256 + lane * 8 < NM);
       cp_async4(&buf.part[k * 32 + lane], pp + k * 32);
     }
     in.lse = d.lse[c];
@@ -439,7 +448,7 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
     if ((j & 31) == 0 && propose) {
       const int cc = c + lane * stride;
       if (cc < d.B) {
-        const int lc = cc / d.M;
+        const int lc = (int)__umulhi((unsigned)cc, d.inv_M);
         const uint4 rw = philox4x32_10_rk(make_uint4(tn, (unsigned)(cc - lc * d.M), (unsigned)lc, 5u), d.rk);
         rwx = rw.x;
         rwy = rw.y;
@@ -452,7 +461,7 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
       load_step_in(d, Zp, prop_slots, NM, c + stride, lane, fst, wbuf[(j + 1) & 1], nxt);
     else
       cp_async_commit();                             // keep one group per chain
-    const int ladder = c / d.M, rg = cur.rung;
+    const int ladder = (int)__umulhi((unsigned)c, d.inv_M), rg = cur.rung;
     int sa = cur.sa, sb = cur.sb;
     const float u = ((float)rx + 0.5f) * 2.3283064365386963e-10f;
     // the draw in case of rejection: lane, chunk, and that chunk's logits
@@ -466,7 +475,7 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
     if (!fst) {
       const float ua = ((float)(unsigned)cur.pr.w + 0.5f) * 2.3283064365386963e-10f;
       const float bound = -s_beta[cur.rung] * (float)cur.pr.y - __int_as_float(cur.pr.z);
-      full = __logf(ua) < bound + 1e-3f;
+      full = __any_sync(0xffffffffu, __logf(ua) < bound + 1e-3f);   // the same on every lane
     }
     const int kp = cur.pr.x & 0xFF, s_old = (cur.pr.x >> 8) & 0xFF;
     bool acc = fst;
@@ -521,12 +530,12 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
         const float lq_rev = row_elem(wr, ei) - lse_p;
         const float log_a = -s_beta[rg] * (float)dE + lq_rev - __int_as_float(cur.pr.z);
         const float ua = ((float)(unsigned)cur.pr.w + 0.5f) * 2.3283064365386963e-10f;
-        acc = log_a >= 0.f || __logf(ua) < log_a;
+        acc = __any_sync(0xffffffffu, log_a >= 0.f || __logf(ua) < log_a);
         if (acc) {
           E += dE;
           unsigned char* sl = d.slots + (size_t)c * d.n;
           if (sa >= 0) sl[lane] = (unsigned char)sa;
-          if (sb >= 0) sl[lane + 32] = (unsigned char)sb;
+          if (kLtTwo<CH> && sb >= 0) sl[lane + 32] = (unsigned char)sb;
           if (lane == 0) {
             d.E[c] = E;
             d.accm[(size_t)ladder * d.M + rg] += 1u;   // one configuration a rung and ladder
@@ -575,7 +584,7 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
         // test whether their move of the drawn chunk is valid there (inside
         // the table, and not the pair's current slot)
         if (lane + 1 == kp) sa = s_old;
-        if (lane + 33 == kp) sb = s_old;
+        if (kLtTwo<CH> && lane + 33 == kp) sb = s_old;
         float cpart[CH];
 #pragma unroll
         for (int k = 0; k < CH; ++k) cpart[k] = sbuf.part[k * 32 + lane];
@@ -584,20 +593,20 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
             (unsigned)((const unsigned short*)&sbuf.crow[rej.kb * 32 + rej.ln])[li] << 16);
         const int m = rej.kb * 256 + rej.ln * 8 + li;
         const int km = m < NM ? mm.k[m] : 1;
-        const int cs = slot_of_lanes(sa, sb, km);
+        const int cs = slot_of<kLtTwo<CH>>(sa, sb, km);
         const bool vi = lane < 8 && m < NM && cs != (int)mm.s[m];
         const int pi = draw_finish(rej, zrej, vi, cur.mx * kLog2e, lane);
         zq = __shfl_sync(0xffffffffu, zrej, pi);
         pick = rej.kb * 256 + rej.ln * 8 + pi;
         lse_c = cur.lse;
       }
-      place_occupancy(sa, sb, d.n, d.delta, s_occ[w], lane);
-      const int kq = mm.k[pick], q_new = mm.s[pick], q_old = slot_of(sa, sb, kq);
+      place_occupancy<kLtTwo<CH>>(sa, sb, d.delta, s_occ[w], lane);
+      const int kq = mm.k[pick], q_new = mm.s[pick], q_old = slot_of<kLtTwo<CH>>(sa, sb, kq);
       const int dk = kq + d.delta;
       const int dEq = move_delta_e(s_occ[w], q_old, dk, q_new);
       unsigned char* ps = prop_slots + (size_t)c * d.n;
       if (sa >= 0) ps[lane] = (unsigned char)(lane + 1 == kq ? q_new : sa);
-      if (sb >= 0) ps[lane + 32] = (unsigned char)(lane + 33 == kq ? q_new : sb);
+      if (kLtTwo<CH> && sb >= 0) ps[lane + 32] = (unsigned char)(lane + 33 == kq ? q_new : sb);
       if (lane == 0) {
         d.prop[c] = make_int4(kq | (q_old << 8) | (q_new << 16), dEq, __float_as_int(zq - lse_c),
                               (int)ry);
@@ -612,7 +621,8 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
       // 8-byte store; a count below 256 is exact in bf16, its float's upper
       // half), the columns of the 2n bins only -- the rest of the row stays
       // 0 from the initial states' input rows
-      for (int col = lane * 4; col < 2 * d.n; col += 128) {
+      const int col = lane * 4;                      // 2n <= 80: one word a lane
+      if (col < 2 * d.n) {
         unsigned h[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -631,6 +641,10 @@ __global__ void __launch_bounds__(256, CH <= 3 ? 3 : 2)
 __global__ void lt_exchange_kernel(LearnedDev d, unsigned t, int count) {
   const int lane = threadIdx.x & 31;
   const int ladder = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  // a programmatic dependent of the step kernel, which writes the energies;
+  // the next forward's first layer may set up meanwhile
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (ladder >= d.L) return;
   const int M = d.M;
   int* lor = d.lor + (size_t)ladder * M;
@@ -696,6 +710,7 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   if (m->variant != variant || m->n != n || M < 2 || M > kPtMaxRungsLearned || L < 1) return SK_EINVAL;
   const int B = L * M, Bp = (B + 127) / 128 * 128, nb = 2 * n + 1;
   if (Bp > m->max_batch) return SK_EINVAL;
+  if ((uint64_t)Bp * (unsigned)M >= 1ULL << 32) return SK_EINVAL;   // beyond inv_M (and any memory)
   int st = check_device();
   if (st) return st;
   std::vector<unsigned long long> ts((size_t)M * nb, 0);
@@ -714,6 +729,7 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   LearnedDev d;
   std::memset(&d, 0, sizeof(d));
   d.n = n; d.delta = m->delta; d.M = M; d.L = L; d.B = B; d.nb = nb; d.NMp = m->NMp;
+  d.inv_M = (unsigned)(((1ULL << 32) + M - 1) / (unsigned)M);
   d.key0 = (unsigned)seed; d.key1 = (unsigned)(seed >> 32);
   for (int r = 0; r < 10; ++r) {
     d.rk[2 * r] = d.key0 + 0x9E3779B9u * (unsigned)r;
@@ -798,34 +814,23 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
                                        iters > 0 && burnin == 0 ? 1 : 0, m->slots, Zb, m->X, m->K1);
     e = cudaGetLastError();
   }
-  // The exchanges of iteration t run on a side stream beside the first layer
-  // of iteration t + 1 (which reads only the input rows and the weights); the
-  // stream joins them before the second layer, ahead of the step kernel of
-  // t + 1 (it reads the rungs and writes the energies they read).
-  cudaStream_t xs = nullptr;
-  cudaEvent_t ev_step = nullptr, ev_exch = nullptr;
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&xs, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_step, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_exch, cudaEventDisableTiming);
-  // Per iteration: layer 1, the join with the previous exchanges, layers 2
-  // and 3 and the step kernel each launched as a programmatic dependent of
-  // the kernel before it (it sets up while that one finishes).
+  // Per iteration: the three layers, the step kernel and the exchanges, each
+  // launched as a programmatic dependent of the kernel before it (it sets up
+  // while that one finishes).  With the exchanges on a second stream, joined by
+  // events before layer 2, an iteration of 131072 chains of n = 20
+  // took 227 us, in line 218 us (and 210 us with the step kernel's 840 for 890
+  // instructions a chain).
   for (uint64_t t = 0; t < iters && e == cudaSuccess; ++t) {
     // the step kernel wrote the input rows
-    e = mlp_forward_dev(*m, Bp, s, true, true, t > 0 ? ev_exch : nullptr, true);
+    e = mlp_forward_dev(*m, Bp, s, true, true, true, t > 0);
     if (e != cudaSuccess) break;
     const bool more = t + 1 < iters;
     e = launch_dependent(lk.step, chain_grid, 256, (size_t)lk.smem, s, d, mt, (unsigned)t, 0,
                          more ? 1 : 0, 0, m->slots, Zb, m->X, m->K1);
-    if (e == cudaSuccess) e = cudaEventRecord(ev_step, s);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(xs, ev_step, 0);
     if (e != cudaSuccess) break;
-    lt_exchange_kernel<<<(L + 3) / 4, 128, 0, xs>>>(d, (unsigned)t,
-                                                    more && t + 1 >= burnin ? 1 : 0);
-    e = cudaEventRecord(ev_exch, xs);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = launch_dependent(lt_exchange_kernel, (L + 3) / 4, 128, (size_t)0, s, d, (unsigned)t,
+                         more && t + 1 >= burnin ? 1 : 0);
   }
-  if (e == cudaSuccess && iters > 0) e = cudaStreamWaitEvent(s, ev_exch, 0);
   if (e == cudaSuccess) {
     const int per = M * nb;
     lt_reduce_kernel<<<(per + 255) / 256, 256, 0, s>>>(d.hist, L, per, out);
@@ -840,10 +845,6 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
-  if (e != cudaSuccess && xs) cudaStreamSynchronize(xs);   // nothing of it left in flight
-  if (ev_step) cudaEventDestroy(ev_step);
-  if (ev_exch) cudaEventDestroy(ev_exch);
-  if (xs) cudaStreamDestroy(xs);
   cudaFree(p);
   if (own) cudaStreamDestroy(s);
   if (e != cudaSuccess) return cuda_status(e);
