@@ -776,11 +776,12 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
 
 // ------------------------------------------------------------ kernel
 
-// One CTA an SM: 24 warps (80 registers a thread), 16 where the rows of the
-// largest orders would not fit beside the tables.
+// One CTA an SM: 20 warps (96 registers a thread; 24 warps of 80 registers: S(20)
+// 448 for 425 ms, n = 16..18 1 % slower), 16 where the rows of the largest
+// orders would not fit beside the tables.
 constexpr int kSpGroup = 4;
 __host__ __device__ constexpr int sp_max_warps(int DELTA, int N) {
-  return sp_quads(DELTA, N) <= 6 ? 24 : 16;
+  return sp_quads(DELTA, N) <= 6 ? 20 : 16;
 }
 
 template <int DELTA, int N, int LB>
