@@ -85,6 +85,49 @@ def alg_ops_per_term(variant, n, nprimes=3):
     return n + (n - g) + 2 * wide + acc
 
 
+SKIP_MIN_N = 13         # smallest order of the zero-skipping walk
+
+
+def nonzero_share(variant, n, samples=200000, seed=1):
+    """Share of the +-1 assignments (sampled) whose correlations at even
+    distance are all nonzero: the terms the zero-skipping walk multiplies."""
+    import numpy as np
+    rng = np.random.default_rng(seed)
+    length = 2 * n + 1 if variant == 2 else 2 * n
+    x = (rng.integers(0, 2, (samples, length), dtype=np.int8) * 2 - 1).astype(np.int8)
+    if variant == 2:
+        x[:, 2 * n - 1] = 0
+    alive = np.ones(samples, dtype=bool)
+    delta = 1 if variant == 1 else 0
+    for d in range(2, n + delta + 1, 2):
+        alive &= (x[:, :-d] * x[:, d:]).sum(axis=1, dtype=np.int32) != 0
+    return float(alive.mean())
+
+
+def skip_ops_per_term(variant, n, share=None):
+    """32-bit integer operations a term of the zero-skipping walk needs: per 32
+    terms and even distance one table word and one OR; for the share of terms
+    that are not zero, n / 4 packed-byte subtractions, n byte extractions, the
+    int32 products inside the groups (factors of even distance halved), two
+    per wide partial product and two per digit accumulated."""
+    delta = 1 if variant == 1 else 0
+    tested = (n + delta) // 2
+    prod = 1
+    for k in range(1, n + 1):
+        d = k + delta
+        bound = max(2 * n - d, 1)
+        prod *= max(bound // 2, 1) if d % 2 == 0 else bound
+    groups = -(-prod.bit_length() // 31)
+    wide = groups * (groups - 1) // 2           # digits 1, 2, .. times the next group
+    nonzero = -(-n // 4) + n + (n - groups) + 2 * wide
+    return 2 * tested / 32 + (nonzero_share(variant, n) if share is None else share) * nonzero
+
+
+def ops_per_term(variant, n):
+    """Operations a term of the walk that counts order n takes."""
+    return skip_ops_per_term(variant, n) if n >= SKIP_MIN_N else alg_ops_per_term(variant, n)
+
+
 # ------------------------------------------------------------------ clocks
 
 class ClockSampler:
@@ -208,7 +251,7 @@ def job_throughput(world, steps, units_per_step, seconds):
 
 def source_hash():
     h = hashlib.sha256()
-    for f in ("sk_exact.cuh", "sk_exact_launch.cuh"):
+    for f in ("sk_exact.cuh", "sk_exact_launch.cuh", "sk_sparse.cuh"):
         with open(os.path.join(ROOT, "paper_1507_00315_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -372,8 +415,8 @@ def run_ie_bench(args, sk, sh):
     algebraic count of Lemma 2.1 on the mid-size workload: each job counted
     both ways (the counts must agree bit for bit), best of `steps` runs of
     each.  Inclusion-exclusion sums 2^{2n} terms, the algebraic count 2^{2n-1}
-    (Lemma 2.2); both walks do the same work per term (n correlation updates,
-    the exact product, one signed accumulate)."""
+    (Lemma 2.2) and skips its zero terms from n = 13 on, which
+    inclusion-exclusion's nonnegative counts hardly have."""
     peak = sk.int32_peak(1)[0]
     out = {}
     for v, n in JOBS:
@@ -389,7 +432,8 @@ def run_ie_bench(args, sk, sh):
             rate = rep["terms"] / (best / 1e3)
             row[name] = {"count": str(c0), "terms": rep["terms"], "kernel_ms": best,
                          "terms_per_s": rate,
-                         "int32_frac": alg_ops_per_term(v, n) * rate / peak}
+                         "int32_frac": (ops_per_term(v, n) if name == "algebraic" else
+                                        alg_ops_per_term(v, n)) * rate / peak}
         assert row["algebraic"]["count"] == row["inclusion_exclusion"]["count"], (v, n, row)
         row["time_ratio_ie_vs_algebraic"] = (row["inclusion_exclusion"]["kernel_ms"] /
                                              row["algebraic"]["kernel_ms"])
@@ -440,7 +484,7 @@ def run_slices_bench(args, sk, sh):
         os.remove(path)
         terms = chunk << m
         rate = terms / (best / 1e3)
-        ops = alg_ops_per_term(v, n)
+        ops = ops_per_term(v, n)
         out[f"{'SLH'[v]}({n})"] = {
             "terms_total": plan["terms"], "walk_bits": m, "items_total": plan["items"],
             "slice_terms": terms, "slice_ms": best, "terms_per_s": rate,
@@ -771,10 +815,11 @@ def run_ours(args, world, rank, local):
     # roofline of the dominant kernel: the largest launch (S(20))
     dom = [x for x in per_launch if x[0] == (0, 20)]
     dom_ms = statistics.mean(x[1] for x in dom)
-    ops = alg_ops_per_term(0, 20) * (1 << 39)
+    per_term = {(v, n): ops_per_term(v, n) for v, n in JOBS}
+    ops = per_term[0, 20] * (1 << 39)
     achieved = ops / (dom_ms / 1e3) / 1e12
     peak = peak_mix / 1e12
-    all_ops = sum(alg_ops_per_term(v, n) * (1 << (2 * n - 1)) for (v, n), _, _ in per_launch)
+    all_ops = sum(per_term[v, n] * (1 << (2 * n - 1)) for (v, n), _, _ in per_launch)
     all_ms = sum(x[1] for x in per_launch)
     line = {
         "metric": METRIC, "value": value, "unit": "terms/s", "n_gpus": world,
@@ -787,8 +832,10 @@ def run_ours(args, world, rank, local):
                    "block_threads": 256, "parallelism": f"{world} replica(s), one GPU each"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
                      "frac": achieved / peak, "traffic": recorded_traffic(),
-                     "kernel": "limb_kernel<0,20> (S(20), 2^39 terms)",
-                     "ops_per_term": alg_ops_per_term(0, 20),
+                     "kernel": "sparse_kernel<0,20,0> (S(20), 2^39 terms, zero terms skipped)",
+                     "ops_per_term": per_term[0, 20],
+                     "dense_ops_per_term": alg_ops_per_term(0, 20),
+                     "nonzero_share": nonzero_share(0, 20),
                      "peak_source": "measured: sk_int32_peak mode 1 (multiply-add / lop3 mix), same run",
                      "imad_pipe_busy_ncu": recorded_imad_busy(),
                      "int32_mad_peak_tops": peak_mad / 1e12,

@@ -40,9 +40,10 @@
 // 60 %, shared-memory pipe 67 % busy, S(17) under ncu): about 945 warp
 // instructions a tile, 600 of them the survivors' evaluation (73 for 32).
 // Whole counts, dense walk (56 instructions a term) and this one: S(20) 1086
-// and 447 ms, hooked n = 18 65.0 and 29.5 ms, mirrored L(19) (Lemmas 2.3 + 2.4)
-// 71.5 and 28.9 ms (one list a tile: 482, 31.4, 35.1 ms).  Below n = 13 no lane
-// block is clear of the low block's partners.
+// and 426 ms, hooked n = 18 65.0 and 28.1 ms, mirrored L(19) (Lemmas 2.3 + 2.4)
+// 71.5 and 25.8 ms; on the way, one list a tile: 482, 31.4, 35.1 ms; 24 warps
+// an SM with 80 registers in place of 20 with 96: 447, 29.5, 28.9 ms.  Below
+// n = 13 no lane block is clear of the low block's partners.
 #pragma once
 #include <cuda_runtime.h>
 
