@@ -12,12 +12,13 @@
 // a fixed order.
 //
 // Persistent and warp-specialised, one CTA (6 warps) per SM:
-//   * every CTA owns one 256-wide column tile of B for the whole launch: its
-//     K/64 slices ([256][64] bf16, 128-byte swizzle) are loaded once by TMA
-//     and stay in shared memory;
+//   * every CTA owns one column tile of B, 256 wide (64 or 128 for batches of
+//     few rows), for the whole launch: its K/64 slices ([256][64] bf16,
+//     128-byte swizzle) are loaded once by TMA, 64 rows a load, and stay in
+//     shared memory;
 //   * warp 0 (one lane) streams the CTA's 128-row tiles of A by TMA, one
 //     [128][64] slice per stage of a 4-deep ring (mbarriers full / empty);
-//   * warp 1 (one lane) issues tcgen05.mma (128 x 256 x 16) for each slice
+//   * warp 1 (one lane) issues tcgen05.mma (128 x tile x 16) for each slice
 //     into one of two 256-column accumulators in tensor memory and commits
 //     them to the ring's "empty" barrier and, per tile, to "acc full";
 //   * warps 2-5 (the epilogue) read the finished accumulator with
@@ -41,6 +42,7 @@ namespace sk {
 constexpr int kTcBM = 128, kTcBN = 256, kTcBK = 64, kTcStages = 4, kTcMaxK = 256;
 constexpr int kTcSliceA = kTcBM * kTcBK * 2;                  // 16 KB
 constexpr int kTcSliceB = kTcBN * kTcBK * 2;                  // 32 KB
+constexpr int kTcBoxN = 64;                                   // rows of B a TMA load brings
 constexpr int kTcStage = 32 * 128;                            // staging: 32 rows x 128 B
 constexpr int kTcThreads = 192;                               // 6 warps
 constexpr int kTcSmem =
@@ -62,6 +64,7 @@ struct TcGemmArgs {
   int ksplit;                     // K ranges (0 or 1: none); needs K / 64 % ksplit == 0
   const __nv_bfloat16* aux;       // kTcEpiMaskBf16: [M][ldaux], C = acc where aux > 0
   int ldaux;
+  int bn;                         // columns of a tile: 64, 128 or 256 (0: 256)
   int nvalid;                     // > 0: only columns < nvalid are wanted (the last column
                                   // tile multiplies and stores that many, rounded up to 16)
   int pdl;                        // launch as a programmatic dependent of the previous kernel
@@ -120,6 +123,14 @@ __device__ __forceinline__ void tc_tma_store(const CUtensorMap* map, unsigned sr
       "r"(x), "r"(y), "r"(src)
       : "memory");
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// The K-major slice of B of one tile, [bn][64] at column x of rows y ..: 64
+// rows (8 KB, eight swizzle groups) a load, one after the other.
+__device__ __forceinline__ void tc_load_b(unsigned dst, const CUtensorMap* map, int x, int y,
+                                          int bn, unsigned mbar) {
+  for (int r = 0; r < bn; r += kTcBoxN)
+    tc_tma_load(dst + (unsigned)(r * kTcBK * 2), map, x, y + r, mbar);
 }
 
 // Shared-memory matrix descriptor, K-major, 128-byte swizzle: 8-row groups
@@ -226,12 +237,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   unsigned char* sB = base;
   unsigned char* sA = STREAMB ? base : base + nkb * kTcSliceB;
   unsigned char* sC = sA + kTcStages * kStageBytes;  // 4 warps x 2 staging buffers
-  const int NT = g.N / kTcBN, MT = g.M / kTcBM;
+  const int bn = g.bn > 0 ? g.bn : kTcBN;
+  const unsigned slice_b = (unsigned)(bn * kTcBK * 2);  // bytes of a B slice that arrive
+  const int NT = g.N / bn, MT = g.M / kTcBM;
   const int groups = gridDim.x / (NT * KS);          // CTAs per (column tile, K range)
   const int nt = blockIdx.x % NT, ks = (blockIdx.x / NT) % KS, m_first = blockIdx.x / (NT * KS);
   const int kb0 = ks * nkb;                          // first K slice of this CTA
   // columns of this CTA's tile that are multiplied (a multiple of 16)
-  const int ncols = g.nvalid > 0 ? min(kTcBN, (g.nvalid - nt * kTcBN + 15) / 16 * 16) : kTcBN;
+  const int ncols = g.nvalid > 0 ? min(bn, (g.nvalid - nt * bn + 15) / 16 * 16) : bn;
   const int my_tiles = (m_first < MT) ? (MT - m_first + groups - 1) / groups : 0;
 
   if (threadIdx.x == 0) {
@@ -268,9 +281,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (STREAMB) {
         tc_arrive(bb);                               // nothing resident to wait for
       } else {
-        tc_expect_tx(bb, (unsigned)(nkb * kTcSliceB));
+        tc_expect_tx(bb, (unsigned)nkb * slice_b);
         for (int kb = 0; kb < nkb; ++kb)
-          tc_tma_load(tc_smem_u32(sB + kb * kTcSliceB), &bmap, (kb0 + kb) * kTcBK, nt * kTcBN, bb);
+          tc_load_b(tc_smem_u32(sB + kb * kTcSliceB), &bmap, (kb0 + kb) * kTcBK, nt * bn, bn, bb);
       }
       // launched as a programmatic dependent (g.pdl): the previous kernel's
       // results (A) only after it has completed; resident weights (B) may
@@ -289,10 +302,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           }
           const unsigned fb = tc_smem_u32(&full_bar[s]);
           unsigned char* stg = sA + s * kStageBytes;
-          tc_expect_tx(fb, (unsigned)kStageBytes);
+          tc_expect_tx(fb, (unsigned)kTcSliceA + (STREAMB ? slice_b : 0u));
           tc_tma_load(tc_smem_u32(stg), &amap, (kb0 + kb) * kTcBK, mt * kTcBM, fb);
           if (STREAMB)
-            tc_tma_load(tc_smem_u32(stg + kTcSliceA), &bmap, (kb0 + kb) * kTcBK, nt * kTcBN, fb);
+            tc_load_b(tc_smem_u32(stg + kTcSliceA), &bmap, (kb0 + kb) * kTcBK, nt * bn, bn, fb);
         }
       }
       if (!ok) atomicOr(g.err, 1u);
@@ -364,20 +377,29 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     unsigned char* stage0 = sC + q * 2 * kTcStage;
     // the bias of this CTA's column tile, staged once (named barrier of the
     // 128 epilogue threads)
-    for (int i = threadIdx.x - 64; i < kTcBN; i += 128)
-      sbias[i] = g.bias ? __ldg(g.bias + nt * kTcBN + i) : 0.f;
+    for (int i = threadIdx.x - 64; i < bn; i += 128)
+      sbias[i] = g.bias ? __ldg(g.bias + nt * bn + i) : 0.f;
     asm volatile("bar.sync 1, 128;" ::: "memory");
     bool ok = true;
     unsigned slab = 0;                               // slabs stored by this warp
     for (int t = 0; t < my_tiles; ++t) {
       const int acc = t & 1;
       const int mt = m_first + t * groups;
+      const int n0 = nt * bn, row0 = mt * kTcBM + q * 32;
+      // the masked epilogue's auxiliary values of the first slab come while
+      // the products run
+      uint4 ax[8];
+      const uint4* ap = nullptr;
+      if constexpr (EPI == kTcEpiMaskBf16) {
+        ap = (const uint4*)(g.aux + (size_t)(row0 + lane) * g.ldaux + n0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) ax[c] = __ldg(ap + c);
+      }
       if (!tc_wait(tc_smem_u32(&accf_bar[acc]), (t >> 1) & 1)) {
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int n0 = nt * kTcBN, row0 = mt * kTcBM + q * 32;
       const int crow0 = ks * g.M + row0;             // a K split's partial goes to its own rows
       if constexpr (EPI != kTcEpiMaskBf16) {
         // software-pipelined: the next slab's accumulator loads are in flight
@@ -413,10 +435,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           unsigned char* st = stage0 + (slab & 1) * kTcStage;
           unsigned v[kCols];
           tc_ld_slab<kCols>(v, tmem + ((unsigned)(q * 32) << 16) + (unsigned)(acc * kTcBN + c0));
-          uint4 ax[8];
-          const uint4* ap = (const uint4*)(g.aux + (size_t)(row0 + lane) * g.ldaux + n0 + c0);
+          if (c0 > 0) {
 #pragma unroll
-          for (int c = 0; c < 8; ++c) ax[c] = __ldg(ap + c);
+            for (int c = 0; c < 8; ++c) ax[c] = __ldg(ap + c0 / 8 + c);
+          }
           asm volatile("tcgen05.wait::ld.sync.aligned;");
           unsigned w[32];                              // this row's 128 bytes of the slab
           // two results at a time, one packed round-to-nearest-even
