@@ -70,7 +70,6 @@ CallScope::CallScope(size_t dbytes, size_t hbytes, void* user_stream)
     err_ = cudaHostAlloc(&set_.hmem, rounded(hbytes), cudaHostAllocDefault);
     if (err_ == cudaSuccess) set_.hcap = rounded(hbytes);
   }
-  drained_ = err_ != cudaSuccess;              // nothing was enqueued
 }
 
 cudaError_t CallScope::drain() {

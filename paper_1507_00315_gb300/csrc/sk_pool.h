@@ -27,8 +27,9 @@ struct CallSet {
 };
 
 // Holds a set for one call.  user_stream: run there instead of the set's own
-// stream.  The destructor waits for the stream where the call did not
-// (`drained` unset) and gives the set back.
+// stream.  The destructor waits for the stream if it was handed out after the
+// last drain() (work may have been enqueued, on an error path too) and gives
+// the set back.
 class CallScope {
  public:
   CallScope(size_t dbytes, size_t hbytes, void* user_stream);
@@ -36,7 +37,11 @@ class CallScope {
   CallScope(const CallScope&) = delete;
   CallScope& operator=(const CallScope&) = delete;
   cudaError_t error() const { return err_; }
-  cudaStream_t stream() const { return user_ ? user_ : set_.stream; }
+  // The stream to enqueue on; take it again after a drain() before new work.
+  cudaStream_t stream() {
+    drained_ = false;
+    return user_ ? user_ : set_.stream;
+  }
   cudaEvent_t e0() const { return set_.e0; }
   cudaEvent_t e1() const { return set_.e1; }
   char* dmem() const { return set_.dmem; }
@@ -48,7 +53,7 @@ class CallScope {
   CallSet set_;
   cudaStream_t user_ = nullptr;
   cudaError_t err_ = cudaSuccess;
-  bool drained_ = false;
+  bool drained_ = true;            // nothing enqueued since
 };
 
 }  // namespace sk
