@@ -541,6 +541,14 @@ void sk_default_primes(uint64_t *out4);
 /* Text for a status code (static storage). */
 const char *sk_strerror(int status);
 
+/* Between calls the library keeps streams, timing events and memory of up to 8
+ * earlier calls a device (at most 32 MiB of device and 32 MiB of pinned host
+ * memory each), so that the next one need not create them; they give way when
+ * an allocation of the library would fail otherwise.  Frees what is idle on
+ * the current device; calls running in other threads keep theirs.  Call it to
+ * hand the memory to another user of the GPU, and before cudaDeviceReset. */
+int sk_release_memory(void);
+
 /* Library version (major * 10000 + minor * 100 + patch). */
 int sk_version(void);
 

@@ -377,6 +377,14 @@ def count_plan(variant, n: int, **kw):
     return rep.as_dict()
 
 
+def release_memory():
+    """sk_release_memory: frees what the library keeps between calls on the
+    current device."""
+    st = lib().sk_release_memory()
+    if st != SK_OK:
+        raise SkolemError(st, "sk_release_memory")
+
+
 def int32_peak(mode: int = 0):
     """sk_int32_peak: (ops per second, ms of the timed launch)."""
     v, ms = ctypes.c_double(), ctypes.c_double()

@@ -19,6 +19,7 @@
 #include "sk_batch.cuh"
 #include "sk_exact_launch.cuh"
 #include "sk_host_common.h"
+#include "sk_pool.h"
 
 SK_DECLARE_BATCH(1) SK_DECLARE_BATCH(2) SK_DECLARE_BATCH(3) SK_DECLARE_BATCH(4)
 SK_DECLARE_BATCH(5) SK_DECLARE_BATCH(6) SK_DECLARE_BATCH(7) SK_DECLARE_BATCH(8)
@@ -155,7 +156,7 @@ int tune_impl(int variant, int n, const sk_batch_opts* o, sk_tune_result* out) {
     own = true;
   }
   ExactScratch* d = nullptr;
-  if (cudaMalloc(&d, sizeof(ExactScratch)) != cudaSuccess) {
+  if (device_malloc((void**)&d, sizeof(ExactScratch)) != cudaSuccess) {
     if (own) cudaStreamDestroy(s);
     return SK_ENOMEM;
   }
@@ -367,7 +368,7 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   double kms_last = 0.0, kms_min = 1e300;
   int launches = 0;
-  e = cudaMalloc(&dbuf, bytes);
+  e = device_malloc((void**)&dbuf, bytes);
   if (e == cudaSuccess) e = cudaHostAlloc(&hbuf, out_bytes, cudaHostAllocDefault);
   if (e == cudaSuccess) e = cudaMemcpy(dbuf, hj.data(), sizeof(BatchJobDev) * njobs, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(dbuf + off_p, &P, sizeof(Primes), cudaMemcpyHostToDevice);

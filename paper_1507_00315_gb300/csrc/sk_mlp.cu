@@ -20,6 +20,7 @@
 #include "sk_gemm_tc.cuh"
 #include "sk_host_common.h"
 #include "sk_mlp.cuh"
+#include "sk_pool.h"
 
 namespace sk {
 
@@ -625,7 +626,7 @@ static cudaError_t bwd_workspace(Mlp& m, int B, BwdSpace (&w)[3]) {
     if (m.bwd_ws) cudaFree(m.bwd_ws);
     m.bwd_ws = nullptr;
     m.bwd_bytes = 0;
-    cudaError_t e = cudaMalloc(&m.bwd_ws, off);
+    cudaError_t e = device_malloc(&m.bwd_ws, off);
     if (e != cudaSuccess) return e;
     m.bwd_bytes = off;
   }
@@ -824,7 +825,7 @@ int mlp_create(int variant, int n, int max_batch, uint64_t seed, Mlp** out) {
   const size_t o_err = off; off = al256(off + 4);
   const size_t o_map = off; off = al256(off + (size_t)m->NMp * 2);
   char* p = nullptr;
-  if (cudaMalloc(&p, off) != cudaSuccess) {
+  if (device_malloc((void**)&p, off) != cudaSuccess) {
     delete m;
     return SK_ENOMEM;
   }
@@ -1104,10 +1105,10 @@ int mlp_train_impl(Mlp& m, const uint8_t* states, uint64_t count, int epochs, in
   cudaStream_t s = nullptr;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMalloc(&dstates, count * m.n);
-  if (e == cudaSuccess) e = cudaMalloc(&didx, count * sizeof(unsigned));
+  if (e == cudaSuccess) e = device_malloc((void**)&dstates, count * m.n);
+  if (e == cudaSuccess) e = device_malloc((void**)&didx, count * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaHostAlloc(&hloss, steps * sizeof(float), cudaHostAllocDefault);
-  if (e == cudaSuccess) e = cudaMalloc(&dloss, steps * sizeof(float));
+  if (e == cudaSuccess) e = device_malloc((void**)&dloss, steps * sizeof(float));
   if (e == cudaSuccess) e = cudaMemcpy(dstates, states, count * m.n, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);

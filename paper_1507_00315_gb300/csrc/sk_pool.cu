@@ -3,6 +3,7 @@
 #include <vector>
 
 #include "sk_exact_launch.cuh"
+#include "sk_host_common.h"
 #include "sk_pool.h"
 
 namespace sk {
@@ -31,7 +32,37 @@ void destroy(CallSet& s) {
 
 size_t rounded(size_t bytes) { return (bytes + 4095) / 4096 * 4096; }
 
+cudaError_t host_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaHostAlloc(p, bytes, cudaHostAllocDefault);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  e = pool_release();
+  return e == cudaSuccess ? cudaHostAlloc(p, bytes, cudaHostAllocDefault) : e;
+}
+
 }  // namespace
+
+cudaError_t pool_release() {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::vector<CallSet> idle;
+  if (dev >= 0 && dev < kMaxDevices) {
+    Pool& p = pool();
+    std::lock_guard<std::mutex> lock(p.mu);
+    idle.swap(p.free_sets[dev]);
+  }
+  for (CallSet& s : idle) destroy(s);
+  return cudaSuccess;
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  e = pool_release();
+  return e == cudaSuccess ? cudaMalloc(p, bytes) : e;
+}
 
 CallScope::CallScope(size_t dbytes, size_t hbytes, void* user_stream)
     : user_((cudaStream_t)user_stream) {
@@ -60,14 +91,14 @@ CallScope::CallScope(size_t dbytes, size_t hbytes, void* user_stream)
     if (set_.dmem) cudaFree(set_.dmem);
     set_.dmem = nullptr;
     set_.dcap = 0;
-    err_ = cudaMalloc(&set_.dmem, rounded(dbytes));
+    err_ = device_malloc((void**)&set_.dmem, rounded(dbytes));
     if (err_ == cudaSuccess) set_.dcap = rounded(dbytes);
   }
   if (err_ == cudaSuccess && set_.hcap < hbytes) {
     if (set_.hmem) cudaFreeHost(set_.hmem);
     set_.hmem = nullptr;
     set_.hcap = 0;
-    err_ = cudaHostAlloc(&set_.hmem, rounded(hbytes), cudaHostAllocDefault);
+    err_ = host_malloc((void**)&set_.hmem, rounded(hbytes));
     if (err_ == cudaSuccess) set_.hcap = rounded(hbytes);
   }
 }
@@ -104,3 +135,5 @@ CallScope::~CallScope() {
 }
 
 }  // namespace sk
+
+extern "C" int sk_release_memory(void) { return sk::cuda_status(sk::pool_release()); }

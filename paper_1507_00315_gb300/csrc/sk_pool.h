@@ -6,7 +6,9 @@
 // from the pool.  A call takes a set of its own and gives it back when it returns,
 // after its stream has drained, so calls of several threads and streams never
 // share one.  At most kPoolSlots sets a device are kept, each with at most
-// kPoolBytes of device and of host memory; the rest is freed at once.
+// kPoolBytes of device and of host memory; the rest is freed at once.  Idle sets
+// never stand in the way of an allocation of the library (device_malloc), and
+// a caller can have them freed (sk_release_memory).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -55,5 +57,11 @@ class CallScope {
   cudaError_t err_ = cudaSuccess;
   bool drained_ = true;            // nothing enqueued since
 };
+
+// Frees the idle sets of the current device.
+cudaError_t pool_release();
+
+// cudaMalloc; where the device is full, once more without the idle sets.
+cudaError_t device_malloc(void** p, size_t bytes);
 
 }  // namespace sk

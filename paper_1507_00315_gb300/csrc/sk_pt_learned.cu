@@ -18,6 +18,7 @@
 
 #include "sk_host_common.h"
 #include "sk_mlp.cuh"
+#include "sk_pool.h"
 #include "sk_pt.cuh"
 
 namespace sk {
@@ -755,7 +756,7 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   const size_t o_ts = off; off = al(off + ts.size() * 8);
   const size_t o_out = off; off = al(off + ((size_t)M * nb + 2 * M) * 8);
   char* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, off);
+  cudaError_t e = device_malloc((void**)&p, off);
   if (e != cudaSuccess) {
     if (own) cudaStreamDestroy(s);
     return SK_ENOMEM;

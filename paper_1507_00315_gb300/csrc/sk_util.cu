@@ -10,6 +10,7 @@
 #include <cstdint>
 
 #include "sk_host_common.h"
+#include "sk_pool.h"
 
 namespace sk {
 
@@ -57,7 +58,7 @@ extern "C" int sk_int32_peak(int mode, double* ops_per_s, double* ms) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   unsigned* sink = nullptr;
-  if (cudaMalloc(&sink, 16) != cudaSuccess) return SK_ENOMEM;
+  if (sk::device_malloc((void**)&sink, 16) != cudaSuccess) return SK_ENOMEM;
   const int threads = 256, blocks = sms * 8;
   const unsigned iters = 4096;
   cudaEvent_t e0, e1;
