@@ -261,7 +261,7 @@ def _variant(v) -> int:
 
 def _rows(flat, k: int):
     """A ctypes array of rows of k words as a list of lists of ints."""
-    return _np().ctypeslib.as_array(flat).reshape(-1, k).tolist()
+    return memoryview(flat).cast("B").cast("Q", (len(flat) // k, k)).tolist()
 
 
 def default_primes():
