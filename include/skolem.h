@@ -129,7 +129,11 @@ typedef struct sk_count_opts {
   int convention;              /* SK_COUNT_REFLECTIONS_IDENTIFIED (default) or
                                   SK_COUNT_ALL */
   int walk_bits;               /* m: Gray-walk bits per work item; 0 -> planner */
-  int block_threads;           /* 32..256, multiple of 32; 0 -> 256 */
+  int block_threads;           /* CTA of the dense Gray walk: 32..256, multiple
+                                  of 32; 0 -> 256.  The zero-skipping walk
+                                  (whole counts and aligned chunks from n = 13
+                                  on) has its own, 640 threads or, from n = 25
+                                  on, 512; work items only bound its chunks */
   int grid;                    /* CTAs; 0 -> SMs x resident CTAs per SM */
   void *stream;                /* cudaStream_t or NULL */
   const char *checkpoint_path; /* NULL: no checkpoint.  Else completed chunks
@@ -156,7 +160,7 @@ typedef struct sk_count_report {
   int walk_bits;               /* m */
   int inner_bits;              /* unrolled Gray bits */
   int arith;                   /* arithmetic form used */
-  int block_threads, grid;
+  int block_threads, grid;     /* of the dense walk; grid 0: one wave */
   uint64_t chunks_total, chunks_done, chunks_resumed;
   int complete;                /* 1 when every chunk is done */
   double kernel_ms;            /* device time of the launches of this call */
@@ -208,7 +212,9 @@ typedef struct sk_batch_opts {
                                      report gives the last and the fastest */
   int autotune;                   /* 1: tune walk width (and block size) per
                                      (variant, n) before the run, untimed */
-  int block_threads;              /* 0 -> 256 or the tuned value */
+  int block_threads;              /* 0 -> 256 or the tuned value; at least 128 in
+                                     a persistent launch with an order of 13 or
+                                     more; one launch per job: as sk_count_opts */
   int walk_bits[SK_MAX_N + 1];    /* per n; 0 -> tuned or planner default */
   void *stream;                   /* cudaStream_t or NULL */
 } sk_batch_opts;

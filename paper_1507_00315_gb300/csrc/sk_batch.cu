@@ -231,6 +231,8 @@ extern "C" int skolem_autotune(int variant, int n, const sk_batch_opts* opts, sk
 namespace sk {
 namespace {
 
+constexpr int kBatchMinSparse = 128;   // threads of a persistent CTA with zero-skipping jobs
+
 struct JobPlan {
   int variant, n, delta, m;
   unsigned long long items, terms;
@@ -319,6 +321,11 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
       max_ws = std::max(max_ws, ws_len(J.delta, J.n));
     }
   }
+  // The warps of a persistent CTA share the zero-skipping walk's 54 KB of
+  // tables: three CTAs an SM at most, so few warps of narrow ones.  S(17), L(17)
+  // and hooked n = 16 at 32 / 64 / 128 / 256 threads: 65.8, 35.7, 21.4, 18.5 ms
+  // (dense walk 38 to 40 ms).
+  if (sparse && mode == SK_BATCH_PERSISTENT && bt < kBatchMinSparse) bt = kBatchMinSparse;
   // persistent grid: SMs x resident CTAs; then the zero-skipping jobs' units
   const size_t smem = (size_t)max_ws * kWsStride +
                       (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kBatchWarp : 0);
@@ -401,7 +408,6 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
           L.P = P;
           L.nprimes = k;
           L.scratch = (ExactScratch*)(dbuf + off_j) + q;
-          L.block_threads = bt;
           L.stream = s;
           r = sparse_launcher(J.delta, J.n, false)(L);
           ++launches;

@@ -379,7 +379,6 @@ static int run_chunk(const Plan& pl, unsigned long long lo, unsigned long long h
     S.P = pl.P;
     S.nprimes = pl.nprimes;
     S.scratch = dscr;
-    S.block_threads = pl.block_threads;
     S.grid = pl.grid;
     S.stream = st;
     e = pl.sparse(S);

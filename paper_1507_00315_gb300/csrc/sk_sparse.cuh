@@ -931,36 +931,34 @@ struct SpLaunch {
   Primes P;
   int nprimes;
   ExactScratch* scratch;
-  int block_threads;
   int grid;                       // 0: SMs x resident blocks
   cudaStream_t stream;
 };
 
+// The CTA size is the walk's own: its warps share 54 KB of tables, so the
+// caller's block size (the dense walk's) would leave SMs short of warps: S(17)
+// at 32 threads 24.9 ms, dense walk 17.1; at 640 threads 7.8 ms.
 template <int DELTA, int N, int LB>
 cudaError_t launch_sparse(const SpLaunch& L) {
   static OccupancyCache occ;
-  const int bt = L.block_threads;
-  if (L.nprimes < 1 || L.nprimes > kMaxPrimes || bt < 32 || bt > 256 || (bt & 31))
-    return cudaErrorInvalidValue;
-  // 256 threads (the default) stand for the widest CTA of this walk
-  constexpr int kWarps = sp_max_warps(DELTA, N);
+  if (L.nprimes < 1 || L.nprimes > kMaxPrimes) return cudaErrorInvalidValue;
+  constexpr int warps = sp_max_warps(DELTA, N);
   constexpr int kArea = sp_warp_bytes(sp_quads(DELTA, N), kSpGroup);
-  const int warps = bt == 256 ? kWarps : bt / 32;
-  const size_t smem = sp_table_bytes(LB) + (size_t)warps * kArea;
+  constexpr int smem = sp_table_bytes(LB) + warps * kArea;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const bool keyed = dev >= 0 && dev < kMaxDevices;
-  int nb = keyed ? occ.per_sm[dev][bt / 32].load(std::memory_order_relaxed) : 0;
-  if (nb <= 0) {                  // first launch of this shape on the device
+  int nb = keyed ? occ.per_sm[dev][0].load(std::memory_order_relaxed) : 0;
+  if (nb <= 0) {                  // first launch on the device
     e = cudaFuncSetAttribute(sparse_kernel<DELTA, N, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sp_table_bytes(LB) + kWarps * kArea);
+                             smem);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, sparse_kernel<DELTA, N, LB>,
                                                         32 * warps, smem);
     if (e != cudaSuccess) return e;
     if (nb <= 0) nb = 1;
-    if (keyed) occ.per_sm[dev][bt / 32].store(nb, std::memory_order_relaxed);
+    if (keyed) occ.per_sm[dev][0].store(nb, std::memory_order_relaxed);
   }
   const unsigned long long wave = (unsigned long long)device_sm_count(dev) * nb;
   SpJob J = L.job;
