@@ -210,8 +210,10 @@ typedef struct sk_batch_opts {
                                      1 launches it directly */
   int repeats;                    /* runs of the whole batch (>= 1; 0 -> 1); the
                                      report gives the last and the fastest */
-  int autotune;                   /* 1: tune walk width (and block size) per
-                                     (variant, n) before the run, untimed */
+  int autotune;                   /* 1: tune block size and, for n <= 12, walk
+                                     width per (variant, n) before the run,
+                                     untimed; the block size of the largest job
+                                     is the batch's */
   int block_threads;              /* 0 -> 256 or the tuned value; at least 128 in
                                      a persistent launch with an order of 13 or
                                      more; one launch per job: as sk_count_opts */
@@ -246,10 +248,11 @@ typedef struct sk_tune_result {
   int candidates;                 /* configurations timed */
 } sk_tune_result;
 
-/* Times candidate walk widths m (planner default and +-2, +-4, within the
- * valid range) and block sizes (128, 256) of the exact-limb kernel for one
- * (variant, n) on the first work items (2^33 terms at most) and returns the
- * fastest.  The result is also cached in the library and used by
+/* Times block sizes (128, 256) and, for n <= 12, candidate walk widths m
+ * (planner default and +-2, +-4, within the valid range) for one (variant, n)
+ * and returns the fastest: the dense walk on the first work items, from n = 13
+ * on the persistent batch's zero-skipping walk on the first 2^31 terms at
+ * most (walk_bits is then the planner's).  The result is also cached in the library and used by
  * skolem_count_batch when opts->autotune is set.  opts may be NULL (only
  * nprimes/primes/stream are read). */
 int skolem_autotune(int variant, int n, const sk_batch_opts *opts, sk_tune_result *out);

@@ -106,6 +106,8 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
 namespace sk {
 namespace {
 
+constexpr int kBatchMinSparse = 128;   // threads of a persistent CTA with zero-skipping jobs
+
 struct Tuned {
   int m = 0, bt = 0;
   double rate = 0.0;
@@ -125,11 +127,93 @@ int batch_primes(const sk_batch_opts* o, int* k, uint64_t* pv, Primes* P) {
 
 int delta_of(int variant) { return variant == SK_LANGFORD ? 1 : 0; }
 
-// Times the exact-form kernel of one (variant, n) on its first items -- one
-// full wave, SMs x 512 resident threads with one item each, so every
-// candidate is timed in the steady state of a long launch -- and keeps the
-// fastest configuration; the default one unless another is at least 3 %
-// faster (single timings of this length vary by about 1 %).
+// Shared memory and full grid (SMs x resident CTAs) of a persistent launch.
+cudaError_t batch_wave(int bt, int max_ws, int sparse, size_t* smem, int* grid) {
+  *smem = (size_t)max_ws * kWsStride +
+          (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kBatchWarp : 0);
+  int dev = 0, nb = 0;
+  cudaGetDevice(&dev);
+  cudaError_t e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       sp_table_bytes(0) + 8 * kBatchWarp +
+                                           ws_len(1, kSparseMinN - 1) * kWsStride);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel, bt, *smem);
+  *grid = device_sm_count(dev) * (nb > 0 ? nb : 1);
+  return e;
+}
+
+// Times the persistent batch of the first tiles of one job of n >= kSparseMinN
+// (2^31 terms at most, about 2 ms) with CTAs of 128 and of 256 threads.
+// The walk width does not enter: the zero-skipping walk takes whole jobs.
+int tune_sparse(int variant, int n, int m0, int k, const Primes& P, cudaStream_t s, Tuned* best,
+                int* cand) {
+  BatchJobDev d;
+  std::memset(&d, 0, sizeof(d));
+  d.pres = position_mask(variant, n);
+  d.m = m0;
+  d.items = 1ULL << (2 * n - 1 - m0);
+  d.code = delta_of(variant) * 32 + n;
+  if (!sp_plain_job(d.pres, delta_of(variant), n, m0, 0, 0, d.items, &d.sp)) return SK_EINVAL;
+  d.sp.range[0].tiles = std::min(d.sp.range[0].tiles, 1ULL << 21);
+  // job | primes | chunk counter | sums
+  const size_t off_p = (sizeof(BatchJobDev) + 255) / 256 * 256;
+  const size_t off_s = off_p + (sizeof(Primes) + 255) / 256 * 256;
+  const size_t bytes = off_s + 256 + sizeof(ExactScratch);
+  CallScope cs(bytes, 0, s);
+  if (cs.error() != cudaSuccess) return cuda_status(cs.error());
+  s = cs.stream();
+  char* dbuf = cs.dmem();
+  cudaError_t e = cudaMemcpyAsync(dbuf + off_p, &P, sizeof(Primes), cudaMemcpyHostToDevice, s);
+  Tuned dflt;
+  for (int bt = 256; bt >= kBatchMinSparse && e == cudaSuccess; bt /= 2) {
+    size_t smem = 0;
+    int grid = 0;
+    e = batch_wave(bt, 0, 1, &smem, &grid);
+    if (e != cudaSuccess) break;
+    sp_split(&d.sp, sp_tiles_per_unit(d.sp.range[0].tiles, (unsigned long long)grid * (bt / 32)));
+    e = cudaMemcpyAsync(dbuf, &d, sizeof(d), cudaMemcpyHostToDevice, s);
+    float ms = 0.f;
+    for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {      // warm, then timed
+      e = cudaMemsetAsync(dbuf + off_s, 0, bytes - off_s, s);
+      if (e == cudaSuccess) e = cudaEventRecord(cs.e0(), s);
+      if (e != cudaSuccess) break;
+      batch_kernel<<<grid, bt, smem, s>>>((const BatchJobDev*)dbuf, 1, d.sp.units,
+                                          (const Primes*)(dbuf + off_p), k,
+                                          (unsigned long long*)(dbuf + off_s),
+                                          (ExactScratch*)(dbuf + off_s + 256), 1);
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaEventRecord(cs.e1(), s);
+      if (e == cudaSuccess) e = cudaEventSynchronize(cs.e1());
+      if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, cs.e0(), cs.e1());
+    }
+    if (e != cudaSuccess) break;
+    ++*cand;
+    const Tuned t = {m0, bt, (double)d.sp.range[0].tiles * 1024.0 / (ms * 1e-3)};
+    if (bt == 256) dflt = *best = t;
+    else if (t.rate >= 1.03 * dflt.rate) *best = t;
+  }
+  if (e == cudaSuccess) e = cs.drain();
+  return cuda_status(e);
+}
+
+int keep_tuned(int delta, int n, const Tuned& best, int cand, sk_tune_result* out) {
+  {
+    std::lock_guard<std::mutex> lock(g_tune_mu);
+    g_tuned[delta][n] = best;
+  }
+  out->walk_bits = best.m;
+  out->block_threads = best.bt;
+  out->terms_per_s = best.rate;
+  out->candidates = cand;
+  return SK_OK;
+}
+
+// Orders below kSparseMinN: times the dense walk of one (variant, n) on its
+// first items -- one full wave, SMs x 512 resident threads with one item each,
+// so every candidate is timed in the steady state of a long launch -- and keeps
+// the fastest configuration; the default one unless another is at least 3 %
+// faster (single timings of this length vary by about 1 %).  Larger orders:
+// tune_sparse, the kernel their batches run.
 int tune_impl(int variant, int n, const sk_batch_opts* o, sk_tune_result* out) {
   if (variant < SK_SKOLEM || variant > SK_HOOKED || n < 1 || n > kMaxN || !out) return SK_EINVAL;
   int k = 0;
@@ -143,6 +227,13 @@ int tune_impl(int variant, int n, const sk_batch_opts* o, sk_tune_result* out) {
   const int mmax = limb_max_m(delta, n) < F ? limb_max_m(delta, n) : F;
   int m0 = default_walk_bits(n);
   if (m0 > mmax) m0 = mmax;
+  if (n >= kSparseMinN) {
+    Tuned best;
+    int cand = 0;
+    st = tune_sparse(variant, n, m0, k, P, (o && o->stream) ? (cudaStream_t)o->stream : nullptr,
+                     &best, &cand);
+    return st ? st : keep_tuned(delta, n, best, cand, out);
+  }
   std::vector<int> ms;
   for (int dm = -4; dm <= 4; dm += 2) {
     const int m = m0 + dm;
@@ -209,16 +300,7 @@ int tune_impl(int variant, int n, const sk_batch_opts* o, sk_tune_result* out) {
   cudaEventDestroy(e1);
   cudaFree(d);
   if (own) cudaStreamDestroy(s);
-  if (st) return st;
-  {
-    std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_tuned[delta][n] = best;
-  }
-  out->walk_bits = best.m;
-  out->block_threads = best.bt;
-  out->terms_per_s = best.rate;
-  out->candidates = cand;
-  return SK_OK;
+  return st ? st : keep_tuned(delta, n, best, cand, out);
 }
 
 }  // namespace
@@ -230,8 +312,6 @@ extern "C" int skolem_autotune(int variant, int n, const sk_batch_opts* opts, sk
 
 namespace sk {
 namespace {
-
-constexpr int kBatchMinSparse = 128;   // threads of a persistent CTA with zero-skipping jobs
 
 struct JobPlan {
   int variant, n, delta, m;
@@ -327,22 +407,10 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   // (dense walk 38 to 40 ms).
   if (sparse && mode == SK_BATCH_PERSISTENT && bt < kBatchMinSparse) bt = kBatchMinSparse;
   // persistent grid: SMs x resident CTAs; then the zero-skipping jobs' units
-  const size_t smem = (size_t)max_ws * kWsStride +
-                      (sparse ? sp_table_bytes(0) + (size_t)(bt / 32) * kBatchWarp : 0);
+  size_t smem = 0;
   int grid = 0;
-  cudaError_t e = cudaSuccess;
-  {
-    int dev = 0, sms = 0, nb = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sp_table_bytes(0) + 8 * kBatchWarp +
-                                 ws_len(1, kSparseMinN - 1) * kWsStride);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_kernel, bt, smem);
-    if (e != cudaSuccess) return cuda_status(e);
-    grid = sms * (nb > 0 ? nb : 1);
-  }
+  cudaError_t e = batch_wave(bt, max_ws, sparse, &smem, &grid);
+  if (e != cudaSuccess) return cuda_status(e);
   const int tpu = sp_tiles_per_unit(tiles, (unsigned long long)grid * (bt / 32));
   unsigned long long chunk = 0;
   for (int r = 0; r < njobs; ++r) {
