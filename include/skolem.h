@@ -424,7 +424,8 @@ int sk_mlp_check(void *model);
 /* The learned tempering run behind pt_estimate_ex with SK_PT_LEARNED, with
  * the outputs of sk_pt_run (no final states).  Needs a model of the same
  * (variant, n) whose max_batch >= L * M rounded up to 128.  Everything runs
- * on one stream; the call returns after it has finished. */
+ * on one stream (with sk_mlp_set_gemm(model, 0) the exchanges run on a second
+ * one, joined to it); the call returns after it has finished. */
 int sk_pt_run_learned(int variant, int n, int M, const double *beta, int L, uint64_t iters,
                       uint64_t burnin, uint64_t seed, const void *model, uint64_t *hist,
                       uint64_t *acc_move, uint64_t *acc_swap);

@@ -524,7 +524,7 @@ cudaError_t gemm_tc(const TcGemmArgs& g, const CUtensorMap& amap, const CUtensor
 // Forward pass for B (multiple of 128) states whose slots are already in
 // m.slots: X, H1, H2 (bf16) and Z (fp32 logits, or bf16 with logits_bf16).
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, bool inputs_ready,
-                            bool dependent, bool first_dependent) {
+                            bool dependent, bool first_dependent, cudaEvent_t before_l2) {
   if (!inputs_ready)
     mlp_inputs_kernel<<<(B + 7) / 8, 256, 0, s>>>(m.slots, B, m.n, m.delta, m.K1, m.X, nullptr,
                                                   nullptr);
@@ -553,6 +553,7 @@ cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16, boo
   g.M = B; g.N = kHidden; g.K = m.K1f; g.A = m.X; g.lda = m.K1; g.B = m.W1; g.ldb = kHidden;
   g.C = m.H1; g.ldc = kHidden; g.bias = m.b1;
   cudaError_t e = gemm<false, false, EPI_BF16_RELU>(g, 1, s);
+  if (e == cudaSuccess && before_l2) e = cudaStreamWaitEvent(s, before_l2, 0);
   if (e != cudaSuccess) return e;
   g.K = kHidden; g.A = m.H1; g.lda = kHidden; g.B = m.W2; g.C = m.H2; g.bias = m.b2;
   e = gemm<false, false, EPI_BF16_RELU>(g, 1, s);

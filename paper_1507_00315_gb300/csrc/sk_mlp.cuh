@@ -93,10 +93,11 @@ __device__ __forceinline__ float warp_sum(float v) {
 // the second and third layers are launched as programmatic dependents of the
 // layer before (they may set up while it finishes); first_dependent: the first
 // layer too, of the stream's previous kernel, which must not have written the
-// weights.
+// weights.  On the mma.sync path every layer is an ordinary launch, and
+// before_l2 is an event the stream waits for between the first and the second.
 cudaError_t mlp_forward_dev(Mlp& m, int B, cudaStream_t s, bool logits_bf16 = false,
                             bool inputs_ready = false, bool dependent = false,
-                            bool first_dependent = false);
+                            bool first_dependent = false, cudaEvent_t before_l2 = nullptr);
 
 // Launch of kernel k as a programmatic dependent of the previous kernel of
 // stream s (it must execute griddepcontrol.wait before it reads what that

@@ -821,17 +821,39 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   // events before layer 2, an iteration of 131072 chains of n = 20
   // took 227 us, in line 218 us (and 210 us with the step kernel's 840 for 890
   // instructions a chain).
+  // On the mma.sync path the layers are ordinary launches that wait for the
+  // exchanges whole, so there these run on a second stream beside the first
+  // layer of the next iteration (it reads only the input rows and the weights),
+  // joined before the second: 60 iterations of 64 ladders x 32 rungs of S(20)
+  // take 2.09 ms so, 2.27 ms in line.
+  cudaStream_t xs = nullptr;
+  cudaEvent_t ev_step = nullptr, ev_exch = nullptr;
+  if (!m->use_tc) {
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&xs, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_step, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_exch, cudaEventDisableTiming);
+  }
   for (uint64_t t = 0; t < iters && e == cudaSuccess; ++t) {
     // the step kernel wrote the input rows
-    e = mlp_forward_dev(*m, Bp, s, true, true, true, t > 0);
+    e = mlp_forward_dev(*m, Bp, s, true, true, true, t > 0, t > 0 ? ev_exch : nullptr);
     if (e != cudaSuccess) break;
     const bool more = t + 1 < iters;
     e = launch_dependent(lk.step, chain_grid, 256, (size_t)lk.smem, s, d, mt, (unsigned)t, 0,
                          more ? 1 : 0, 0, m->slots, Zb, m->X, m->K1);
     if (e != cudaSuccess) break;
-    e = launch_dependent(lt_exchange_kernel, (L + 3) / 4, 128, (size_t)0, s, d, (unsigned)t,
-                         more && t + 1 >= burnin ? 1 : 0);
+    const int count = more && t + 1 >= burnin ? 1 : 0;
+    if (!xs) {
+      e = launch_dependent(lt_exchange_kernel, (L + 3) / 4, 128, (size_t)0, s, d, (unsigned)t, count);
+      continue;
+    }
+    e = cudaEventRecord(ev_step, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(xs, ev_step, 0);
+    if (e != cudaSuccess) break;
+    lt_exchange_kernel<<<(L + 3) / 4, 128, 0, xs>>>(d, (unsigned)t, count);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaEventRecord(ev_exch, xs);
   }
+  if (e == cudaSuccess && xs && iters > 0) e = cudaStreamWaitEvent(s, ev_exch, 0);
   if (e == cudaSuccess) {
     const int per = M * nb;
     lt_reduce_kernel<<<(per + 255) / 256, 256, 0, s>>>(d.hist, L, per, out);
@@ -846,6 +868,10 @@ int pt_learned_run(int variant, int n, int M, const double* beta, int L, uint64_
   if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
+  if (e != cudaSuccess && xs) cudaStreamSynchronize(xs);   // nothing of it left in flight
+  if (ev_step) cudaEventDestroy(ev_step);
+  if (ev_exch) cudaEventDestroy(ev_exch);
+  if (xs) cudaStreamDestroy(xs);
   cudaFree(p);
   if (own) cudaStreamDestroy(s);
   if (e != cudaSuccess) return cuda_status(e);
