@@ -123,9 +123,21 @@ def skip_ops_per_term(variant, n, share=None):
     return 2 * tested / 32 + (nonzero_share(variant, n) if share is None else share) * nonzero
 
 
+SPARSE_THREADS = 640       # CTA of the zero-skipping walk up to n = 24
+RECORD_BYTES = 72          # a launch's record: chunk counter, two sums for each of four moduli
+
+
 def ops_per_term(variant, n):
     """Operations a term of the walk that counts order n takes."""
     return skip_ops_per_term(variant, n) if n >= SKIP_MIN_N else alg_ops_per_term(variant, n)
+
+
+def slice_ops_per_term(variant, n, bits):
+    """The same for an aligned slice of 2^bits terms of the count: the
+    zero-skipping walk's tiles need 10 + n + delta of its variables to vary;
+    a smaller slice takes the dense walk."""
+    tiles = n >= SKIP_MIN_N and bits >= 10 + n + (1 if variant == 1 else 0)
+    return skip_ops_per_term(variant, n) if tiles else alg_ops_per_term(variant, n)
 
 
 # ------------------------------------------------------------------ clocks
@@ -484,7 +496,7 @@ def run_slices_bench(args, sk, sh):
         os.remove(path)
         terms = chunk << m
         rate = terms / (best / 1e3)
-        ops = ops_per_term(v, n)
+        ops = slice_ops_per_term(v, n, (chunk << m).bit_length() - 1)
         out[f"{'SLH'[v]}({n})"] = {
             "terms_total": plan["terms"], "walk_bits": m, "items_total": plan["items"],
             "slice_terms": terms, "slice_ms": best, "terms_per_s": rate,
@@ -829,7 +841,7 @@ def run_ours(args, world, rank, local):
         "config": {"workload": WORKLOAD, "jobs": [f"{'SL'[v]}({n})" for v, n in JOBS],
                    "moduli": 3, "l2": "flushed between steps (512 MiB write)",
                    "walk_bits": {f"{'SL'[v]}({n})": r["walk_bits"] for (v, n), _, r in per_launch[:len(JOBS)]},
-                   "block_threads": 256, "parallelism": f"{world} replica(s), one GPU each"},
+                   "block_threads": SPARSE_THREADS, "parallelism": f"{world} replica(s), one GPU each"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
                      "frac": achieved / peak, "traffic": recorded_traffic(),
                      "kernel": "sparse_kernel<0,20,0> (S(20), 2^39 terms, zero terms skipped)",
@@ -841,7 +853,7 @@ def run_ours(args, world, rank, local):
                      "int32_mad_peak_tops": peak_mad / 1e12,
                      "all_launches_frac": (all_ops / (all_ms / 1e3) / 1e12) / peak},
         "e2e": {"value": e2e, "unit": "terms/s", "h2d_bytes_per_step": 0,
-                "d2h_bytes_per_step": 48 * len(JOBS)},
+                "d2h_bytes_per_step": RECORD_BYTES * len(JOBS)},
         "gpu_launches": args.steps * len(JOBS),
         "clocks": clk,
     }
