@@ -140,6 +140,12 @@ def slice_ops_per_term(variant, n, bits):
     return skip_ops_per_term(variant, n) if tiles else alg_ops_per_term(variant, n)
 
 
+def slice_items(items, m, bits):
+    """Work items of a slice of 2^bits terms, m walk bits each: the whole
+    count's where that is smaller."""
+    return min(items, 1 << max(0, bits - m))
+
+
 # ------------------------------------------------------------------ clocks
 
 class ClockSampler:
@@ -483,7 +489,7 @@ def run_slices_bench(args, sk, sh):
         plan = sk.count_plan(v, n, nprimes=4, checkpoint=path, symmetry=sym)
         m = min(plan["walk_bits"], max(plan["inner_bits"], args.slice_bits - 17))
         plan = sk.count_plan(v, n, nprimes=4, checkpoint=path, symmetry=sym, walk_bits=m)
-        chunk = 1 << max(0, args.slice_bits - m)
+        chunk = slice_items(plan["items"], m, args.slice_bits)
         best = None
         for rep_i in range(2):                  # first call warms the kernel up
             if os.path.exists(path):

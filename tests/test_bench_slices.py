@@ -12,3 +12,11 @@ def test_operations_of_a_slice():
         want = bench.skip_ops_per_term(variant, n) if skips else bench.alg_ops_per_term(variant, n)
         assert bench.slice_ops_per_term(variant, n, bits) == want
     assert bench.alg_ops_per_term(1, 31) == 92 and bench.skip_ops_per_term(1, 31) < 13
+
+
+def test_a_slice_is_no_larger_than_the_count():
+    # S(21) with Lemma 2.4: 2^26 items of 2^14 terms (a 2^42-term slice had
+    # been timed over the count's 2^40 terms and booked whole)
+    assert bench.slice_items(1 << 26, 14, 42) == 1 << 26
+    assert bench.slice_items(1 << 26, 14, 38) == 1 << 24
+    assert bench.slice_items(1 << 20, 25, 22) == 1
