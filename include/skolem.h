@@ -45,7 +45,8 @@ enum {
   SK_ERANGE = -2,     /* the moduli cannot represent the value */
   SK_ECUDA = -3,      /* CUDA error or no usable device */
   SK_ENOMEM = -4,     /* device or host allocation failed */
-  SK_ETIMEOUT = -5,   /* a bounded device loop gave up (error word set) */
+  SK_ETIMEOUT = -5,   /* a bounded wait of a network kernel gave up (error
+                         word set; sk_mlp_check) */
   SK_EMISMATCH = -6,  /* a consistency check failed (check prime, 2^{2n-1}
                          divisibility, sign, parity of the count) */
   SK_ECKPT = -7       /* checkpoint file unreadable, corrupt or for another job */
@@ -59,9 +60,9 @@ enum { SK_COUNT_REFLECTIONS_IDENTIFIED = 0, SK_COUNT_ALL = 1 };
 /* Largest n with a compiled exact kernel.  The position set of every variant
  * fits one 64-bit mask up to n = 31 (hooked Skolem spans 2n+1 = 63
  * positions), and the three 62-bit moduli (M ~ 2^186) hold the signed sum
- * C 2^{2n-1} with room to spare (|H| < 2^146 at n = 31).  Counting the
- * 2^{2n-1} terms of n >= 26 takes GPU-days; the work-item calls below reach
- * every order. */
+ * C 2^{2n-1} with room to spare (|H| < 2^146 at n = 31).  A whole count takes
+ * GPU-hours from n = 26 and GPU-days from n = 29 on; the work-item calls below
+ * reach every order. */
 #define SK_MAX_N 31
 
 /* Arithmetic form of the term products (both give identical residues).
@@ -144,8 +145,7 @@ typedef struct sk_count_opts {
   uint64_t max_chunks;         /* stop (status SK_OK, report->complete = 0)
                                   after this many new chunks; 0 = no limit */
   int arith;                   /* SK_ARITH_LIMBS (default) or SK_ARITH_MONTGOMERY */
-  int symmetry;                /* SK_SYMMETRY_NEGATION (default) or
-                                  SK_SYMMETRY_NEGATION_EVEN */
+  int symmetry;                /* SK_SYMMETRY_*; default SK_SYMMETRY_NEGATION */
 } sk_count_opts;
 
 typedef struct sk_count_report {
@@ -195,8 +195,9 @@ int skolem_count_ex(int variant, int n, const sk_count_opts *opts, sk_u128 *out,
 typedef struct sk_job { int variant; int n; } sk_job;
 
 /* SK_BATCH_PERSISTENT: every job in one persistent launch (captured in a CUDA
- * graph unless no_graph) pulling 32-item chunks from a device queue, largest
- * job first.  SK_BATCH_PER_JOB: one launch per job, back to back on the
+ * graph unless no_graph) pulling chunks from a device queue, largest job
+ * first: 32 work items of the dense walk below n = 13, from there on up to 128
+ * tiles of 2^10 terms of the zero-skipping walk.  SK_BATCH_PER_JOB: one launch per job, back to back on the
  * stream (the baseline). */
 enum { SK_BATCH_PERSISTENT = 0, SK_BATCH_PER_JOB = 1 };
 
@@ -227,7 +228,8 @@ typedef struct sk_batch_report {
   double wall_ms;                 /* host time of the whole call */
   double prepare_ms;              /* planning, tuning, graph capture */
   uint64_t terms;                 /* sum over jobs of 2^{2n-1} */
-  uint64_t chunks;                /* 32-item chunks of the queue */
+  uint64_t chunks;                /* 32-item chunks of the jobs' work items (the
+                                     queue's own below n = 13) */
   int launches;                   /* kernel launches per repeat */
   int grid, block_threads;
 } sk_batch_report;

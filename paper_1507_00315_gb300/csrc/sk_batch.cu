@@ -2,14 +2,15 @@
 //
 // skolem_count_batch runs many exact-count jobs (variant x n) in one
 // persistent launch captured in a CUDA graph: jobs are laid end to end in a
-// space of 32-item chunks, largest job first (longest-processing-time order),
+// space of chunks (32 work items of the dense walk, a unit of tiles of the
+// zero-skipping walk), largest job first (longest-processing-time order),
 // every warp pulls the next chunk from a device counter, finds its job by
 // binary search over the chunk offsets, and runs that job's compiled walk.  A
-// warp keeps its residues while it stays on one job and flushes them into the
-// job's slots (modular CAS add) when it moves on.  The same jobs can instead
-// run as one launch per job (SK_BATCH_PER_JOB), the baseline it is measured
-// against.  skolem_autotune times candidate walk widths and block sizes for
-// one (variant, n) on a fixed number of terms and keeps the fastest.
+// warp keeps its residues while it stays on one job and adds them to the job's
+// sums (warp_flush) when it moves on.  The same jobs can instead run as one
+// launch per job (SK_BATCH_PER_JOB), the baseline it is measured against.
+// skolem_autotune times block sizes, and walk widths of the dense walk, for
+// one (variant, n) and keeps the fastest.
 #include <algorithm>
 #include <chrono>
 #include <cstring>

@@ -477,8 +477,9 @@ static cudaError_t tc_attributes(int* dev_out) {
 // one tile's latency (four 64-column slabs of epilogue one after the other), so
 // it is cut into 128 or 64 columns as long as every CTA has a tile of its own:
 // 4096 rows x 256 columns on 128 SMs instead of 32.  A call of 16 training
-// steps at 4096 rows (n = 20): 2.39 ms with 256 columns, 2.26 ms so; the logits
-// of 5000 states (L(24), 80 CTAs for 40) 171 and 151 us.  The narrowed last
+// steps at 4096 rows (n = 20): 2.39 ms with 256 columns, 2.26 ms so (2.09 and
+// 1.98 on another GPU); the logits of 5000 states (L(24), 80 CTAs for 40) 171 and
+// 151 us, runs of either differing by up to 28 %.  The narrowed last
 // tile (nvalid) and a K split keep 256 columns: they have CTAs enough.
 template <int EPI, bool STREAMB>
 cudaError_t gemm_tc_launch(const TcGemmArgs& g0, const CUtensorMap& amap, const CUtensorMap& bmap,

@@ -7,7 +7,7 @@
 // synchronisation cudaFree implies.  This entry point runs the same
 // Gray-code kernel as skolem_item_residues (exact form), but its device
 // scratch -- the
-// launch record (work counter, residue slots, error word) and the per-item
+// launch record (work counter, residue sums) and the per-item
 // staging of the residues before they are copied to the caller's host
 // buffer -- lives in one file-scope __device__ array of fixed size, which
 // every GPU that loads the library holds until the process exits.  It creates

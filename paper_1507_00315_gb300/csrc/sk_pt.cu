@@ -181,9 +181,11 @@ __device__ __forceinline__ void pt_step(const PtLane<GEN>& S, const uint4 wc, co
 
 // Bound by issue and the multiply pipe (65 and 70 % busy under ncu, 135 warp
 // instructions an iteration, 40 of them Philox): 32 rungs x 4096 ladders of
-// S(20) in 711 ns an iteration; with two-role exchanges, 64-bit thresholds and
-// unpredicated stores (165 instructions) 853 ns.  64 rungs of L(32): 1601 and
-// 1864 ns; 256 ladders, bound by one iteration's latency, 221 and 272 ns.  One
+// S(20) in 707 ns an iteration; with two-role exchanges, 64-bit thresholds and
+// unpredicated stores (165 instructions) 846 ns.  64 rungs of L(32): 1544 and
+// 1804 ns (multiply pipe 59 %, issue 64 %; registers and shared memory both hold
+// 7 CTAs an SM, so 4096 ladders take two waves); 256 ladders of 32 rungs, bound by
+// one iteration's latency, 207 and 256 ns; round trips counted 856 and 966 ns.  One
 // ladder a CTA, for an even spread over the SMs, measured the same.
 //
 // W warps = one ladder (W = 1: up to 32 rungs, W = 2: up to 64); persistent

@@ -36,13 +36,13 @@
 // one list, so that few evaluations run part empty; the tiles' a rows wait in
 // shared memory, where the 32 entries of an evaluation read few of them.
 //
-// Bound by instruction issue (82 % of the issue slots, ALU 69 %, multiply pipe
-// 60 %, shared-memory pipe 67 % busy, S(17) under ncu): about 945 warp
-// instructions a tile, 600 of them the survivors' evaluation (73 for 32).
+// Bound by instruction issue (82 % of the issue slots, ALU 70 %, multiply pipe
+// 58 %, shared-memory pipe 70 % busy, S(18) under ncu): 857 warp instructions a
+// tile (928 at n = 17), about 600 of them the survivors' evaluation (73 for 32).
 // Whole counts, dense walk (56 instructions a term) and this one: S(20) 1086
 // and 426 ms, hooked n = 18 65.0 and 28.1 ms, mirrored L(19) (Lemmas 2.3 + 2.4)
-// 71.5 and 25.8 ms; on the way, one list a tile: 482, 31.4, 35.1 ms; 24 warps
-// an SM with 80 registers in place of 20 with 96: 447, 29.5, 28.9 ms.  Below
+// 71.5 and 25.8 ms; on the way, one list a tile: 482, 31.4, 35.1 ms.  (24 warps
+// an SM with 80 registers in place of 20 with 96: 447, 28.2, 28.9 ms.)  Below
 // n = 13 no lane block is clear of the low block's partners.
 #pragma once
 #include <cuda_runtime.h>
@@ -777,9 +777,10 @@ __device__ __forceinline__ Res4 sparse_unit(const SpJob* Jp, unsigned long long 
 
 // ------------------------------------------------------------ kernel
 
-// One CTA an SM: 20 warps (96 registers a thread; 24 warps of 80 registers: S(20)
-// 448 for 425 ms, n = 16..18 1 % slower), 16 where the rows of the largest
-// orders would not fit beside the tables.
+// One CTA an SM: 20 warps (96 registers a thread; 24 warps of 80 registers, kernel
+// time: S(20) 447.1 for 425.4 ms, S(17) 7.87 for 7.79, S(18) 28.2 for 28.0, L(19)
+// with Lemmas 2.3 + 2.4 28.9 for 25.7, but L(20) 444.4 for 445.4), 16 where the
+// rows of the largest orders would not fit beside the tables.
 constexpr int kSpGroup = 4;
 __host__ __device__ constexpr int sp_max_warps(int DELTA, int N) {
   return sp_quads(DELTA, N) <= 6 ? 20 : 16;
