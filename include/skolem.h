@@ -215,9 +215,9 @@ typedef struct sk_batch_opts {
                                      width per (variant, n) before the run,
                                      untimed; the block size of the largest job
                                      is the batch's */
-  int block_threads;              /* 0 -> 256 or the tuned value; at least 128 in
-                                     a persistent launch with an order of 13 or
-                                     more; one launch per job: as sk_count_opts */
+  int block_threads;              /* 0 -> 256 or the tuned value; a value given
+                                     here counts for the dense walk: a persistent
+                                     launch with an order of 13 or more has 256 */
   int walk_bits[SK_MAX_N + 1];    /* per n; 0 -> tuned or planner default */
   void *stream;                   /* cudaStream_t or NULL */
 } sk_batch_opts;

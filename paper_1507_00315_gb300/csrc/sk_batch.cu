@@ -107,8 +107,6 @@ __global__ void __launch_bounds__(256, SK_EXACT_MIN_BLOCKS)
 namespace sk {
 namespace {
 
-constexpr int kBatchMinSparse = 128;   // threads of a persistent CTA with zero-skipping jobs
-
 struct Tuned {
   int m = 0, bt = 0;
   double rate = 0.0;
@@ -166,7 +164,7 @@ int tune_sparse(int variant, int n, int m0, int k, const Primes& P, cudaStream_t
   char* dbuf = cs.dmem();
   cudaError_t e = cudaMemcpyAsync(dbuf + off_p, &P, sizeof(Primes), cudaMemcpyHostToDevice, s);
   Tuned dflt;
-  for (int bt = 256; bt >= kBatchMinSparse && e == cudaSuccess; bt /= 2) {
+  for (int bt = 256; bt >= 128 && e == cudaSuccess; bt /= 2) {
     size_t smem = 0;
     int grid = 0;
     e = batch_wave(bt, 0, 1, &smem, &grid);
@@ -405,8 +403,9 @@ int batch_impl(const sk_job* jobs, int njobs, const sk_batch_opts* o, sk_u128* o
   // The warps of a persistent CTA share the zero-skipping walk's 54 KB of
   // tables: three CTAs an SM at most, so few warps of narrow ones.  S(17), L(17)
   // and hooked n = 16 at 32 / 64 / 128 / 256 threads: 65.8, 35.7, 21.4, 18.5 ms
-  // (dense walk 38 to 40 ms).
-  if (sparse && mode == SK_BATCH_PERSISTENT && bt < kBatchMinSparse) bt = kBatchMinSparse;
+  // (dense walk 38 to 40 ms); orders of 16 at 128 threads 7.0, at 256 4.7 ms.  So
+  // a size given by the caller counts for the dense walk's batches only.
+  if (sparse && mode == SK_BATCH_PERSISTENT && o && o->block_threads) bt = 256;
   // persistent grid: SMs x resident CTAs; then the zero-skipping jobs' units
   size_t smem = 0;
   int grid = 0;
